@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 
 #include "rope_internal.h"
+#include "rope_window_sum.cuh"
 
 namespace rope {
 
@@ -120,8 +121,7 @@ __global__ void features_kernel(DevIndex ix, const uint8_t* __restrict__ seqs, c
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int wpb = blockDim.x >> 5;
-  float2* acc = feat_acc + (size_t)warp * ix.D;
-  const int n_loc = ix.N - ix.s + 1;
+  float2* stage = feat_acc + (size_t)warp * window_sum_smem(ix.m, ix.D);
   const int D = ix.D;
   for (int64_t r = (int64_t)blockIdx.x * wpb + warp; r < n_reads; r += (int64_t)gridDim.x * wpb) {
     const float* x = emb_f32 + (size_t)r * 2 * D;
@@ -133,23 +133,7 @@ __global__ void features_kernel(DevIndex ix, const uint8_t* __restrict__ seqs, c
         for (int f = lane; f < F; f += 32) row[f] = 0.f;
         continue;
       }
-      for (int g = lane; g < D; g += 32) acc[g] = make_float2(0.f, 0.f);
-      __syncwarp();
-      for (int loc0 = 0; loc0 < n_loc; loc0 += 32) {
-        const int loc = loc0 + lane;
-        const uint32_t b = loc < n_loc ? bin_at(ix.packed, w0 + loc, ix.s, ix.map_lsb) : 0u;
-        const int cnt = min(32, n_loc - loc0);
-        for (int jj = 0; jj < cnt; ++jj) {
-          const uint32_t bj = __shfl_sync(0xffffffffu, b, jj);
-          if (lane < ix.m) {
-            const float2 ph = ix.phase[lane * n_loc + loc0 + jj];
-            float2& v = acc[lane * ix.nb + bj];
-            v.x += ph.x;
-            v.y += ph.y;
-          }
-          __syncwarp();
-        }
-      }
+      const float2* acc = window_direct_sum(ix, w0, stage);
       for (int k = 0; k < ix.m; ++k) {
         float re = 0.f, im = 0.f, C = 0.f;
         for (int b = lane; b < ix.nb; b += 32) {
@@ -224,7 +208,7 @@ cudaError_t launch_features(const DevIndex& ix, const uint8_t* seqs, const int64
   const int wpb = 8;
   int64_t blocks = (n_reads + wpb - 1) / wpb;
   if (blocks > 152 * 32) blocks = 152 * 32;
-  features_kernel<<<(unsigned)blocks, wpb * 32, (size_t)wpb * ix.D * sizeof(float2), st>>>(
+  features_kernel<<<(unsigned)blocks, wpb * 32, (size_t)wpb * window_sum_smem(ix.m, ix.D) * sizeof(float2), st>>>(
       ix, seqs, offsets, emb_f32, norms, cand_win, cand_score, n_reads, K, F, X);
   return cudaGetLastError();
 }
