@@ -6,7 +6,10 @@
 // The paper has no reranker; it relates fidelity to Levenshtein distance (§1,
 // §2.4 fitting curve) and thresholds fidelities per fragment (§3.3, §3.5).
 // This network learns that relation from the scan's own score features.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "rope_internal.h"
 #include "rope_window_sum.cuh"
@@ -220,117 +223,217 @@ __device__ __forceinline__ float gelu_grad_f(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.3989422804014327f * expf(-0.5f * z * z);
 }
 
-// Forward: one thread per sample; BF16 weights staged in shared memory as FP32.
-// pre[s][j] is stored when `pre` is non-null (training), and with targets the
-// per-sample residual gradient dy = 2 (y - t) / B and squared error.
+// Forward: a block takes 32 samples, a lane per sample, and each of its warps a
+// share of the hidden units; the BF16 weights are staged in shared memory as
+// FP32 rows padded with zeros to FP (features rounded up to 8), read as float4
+// broadcasts. pre[j][s] is stored when `pre` is non-null (training; unit-major,
+// so stores here and loads in the backward pass are whole lines), and with
+// targets the per-sample residual gradient dy = 2 (y - t) / B and squared error.
 // Sample s of the batch is row idx[s] of X and t (row s when idx is null).
-__global__ void mlp_forward_kernel(MlpWeights w, const float* __restrict__ X, const int64_t* __restrict__ idx,
-                                   int64_t B, float* __restrict__ y, float* __restrict__ pre,
-                                   const float* __restrict__ t, float* __restrict__ dy, float* __restrict__ sq) {
-  extern __shared__ float mlp_smem[];
-  float* W1 = mlp_smem;                  // H x F
-  float* b1 = W1 + w.H * w.F;            // H
-  float* w2 = b1 + w.H;                  // H
-  for (int i = threadIdx.x; i < w.H * w.F; i += blockDim.x) W1[i] = __bfloat162float(w.W1[i]);
+// A training batch (4,096 samples) is latency: with a thread per sample it ran
+// on 32 SMs, 128 units one after another.
+constexpr int kMlpWarps = 4;
+
+template <int FP>
+__global__ void __launch_bounds__(32 * kMlpWarps)
+    mlp_forward_kernel(MlpWeights w, const float* __restrict__ X, const int64_t* __restrict__ idx, int64_t B,
+                       float* __restrict__ y, float* __restrict__ pre, const float* __restrict__ t,
+                       float* __restrict__ dy, float* __restrict__ sq) {
+  extern __shared__ __align__(16) float mlp_smem[];
+  __shared__ float xt[32][FP + 1];
+  __shared__ int64_t rows[32];
+  __shared__ float part[kMlpWarps][32];
+  float* W1 = mlp_smem;       // H x FP
+  float* b1 = W1 + w.H * FP;  // H
+  float* w2 = b1 + w.H;       // H
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < w.H * FP; i += blockDim.x) {
+    const int j = i / FP, f = i - j * FP;
+    W1[i] = f < w.F ? __bfloat162float(w.W1[j * w.F + f]) : 0.f;
+  }
   for (int i = threadIdx.x; i < w.H; i += blockDim.x) {
     b1[i] = w.b1[i];
     w2[i] = __bfloat162float(w.w2[i]);
   }
-  __syncthreads();
   const float b2 = w.b2[0];
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < B; s += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = idx ? idx[s] : s;
-    float xs[kMaxFeatures];
+  const int j_lo = w.H * warp / kMlpWarps, j_hi = w.H * (warp + 1) / kMlpWarps;
+  for (int64_t s0 = (int64_t)blockIdx.x * 32; s0 < B; s0 += (int64_t)gridDim.x * 32) {
+    const int n = (int)min((int64_t)32, B - s0);
+    if (threadIdx.x < 32) rows[lane] = lane < n ? (idx ? idx[s0 + lane] : s0 + lane) : 0;
+    __syncthreads();  // (the weights too, the first time)
+    for (int i = threadIdx.x; i < 32 * FP; i += blockDim.x) {
+      const int q = i / FP, f = i - q * FP;
+      xt[q][f] = q < n && f < w.F ? X[rows[q] * w.F + f] : 0.f;
+    }
+    __syncthreads();
+    float xs[FP];
 #pragma unroll
-    for (int f = 0; f < kMaxFeatures; ++f) xs[f] = f < w.F ? X[row * w.F + f] : 0.f;
-    float acc = b2;
-    for (int j = 0; j < w.H; ++j) {
+    for (int f = 0; f < FP; ++f) xs[f] = xt[lane][f];
+    const int64_t s = s0 + lane;
+    float acc = 0.f;
+#pragma unroll 2
+    for (int j = j_lo; j < j_hi; ++j) {
+      const float4* row = reinterpret_cast<const float4*>(W1 + j * FP);
       float z = b1[j];
 #pragma unroll
-      for (int f = 0; f < kMaxFeatures; ++f)
-        if (f < w.F) z = fmaf(W1[j * w.F + f], xs[f], z);
-      if (pre) pre[s * w.H + j] = z;
+      for (int f = 0; f < FP; f += 4) {
+        const float4 v = row[f / 4];
+        z = fmaf(v.x, xs[f], z);
+        z = fmaf(v.y, xs[f + 1], z);
+        z = fmaf(v.z, xs[f + 2], z);
+        z = fmaf(v.w, xs[f + 3], z);
+      }
+      if (pre && lane < n) pre[(int64_t)j * B + s] = z;
       acc = fmaf(w2[j], gelu_f(z), acc);
     }
-    if (y) y[s] = acc;
-    if (t) {
-      const float r = acc - t[row];
-      dy[s] = 2.0f * r / (float)B;
-      sq[s] = r * r;
+    part[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && lane < n) {
+      float v = b2;
+#pragma unroll
+      for (int q = 0; q < kMlpWarps; ++q) v += part[q][lane];
+      if (y) y[s] = v;
+      if (t) {
+        const float r = v - t[rows[lane]];
+        dy[s] = 2.0f * r / (float)B;
+        sq[s] = r * r;
+      }
     }
+    __syncthreads();  // rows, xt and part are free for the next samples
   }
 }
 
-// Backward: one block per hidden unit j; its threads split the samples and the
-// block reduces in a fixed order (deterministic):
-//   dW1[j][f] = sum_s dy_s w2_j GELU'(pre_sj) x_sf,  db1[j] = sum_s dy_s w2_j GELU'(pre_sj)
-//   dw2[j]    = sum_s dy_s GELU(pre_sj);  block H also forms db2 = sum_s dy_s and the loss.
+// Backward:
+//   dW1[j][f] = sum_s dy_s w2_j GELU'(pre_js) x_sf,  db1[j] = sum_s dy_s w2_j GELU'(pre_js)
+//   dw2[j]    = sum_s dy_s GELU(pre_js);  db2 = sum_s dy_s, and the loss.
+// A cluster of kBwdSplit blocks takes kBwdUnits hidden units, its blocks every
+// kBwdSplit-th tile of 32 samples: per tile the block forms dz (a warp per unit,
+// a lane per sample) and stages the samples' rows, then each warp adds 4 units x
+// FP/4 features with a lane per sample; the next tile's loads are in flight
+// meanwhile. Lanes, then the cluster's blocks (through distributed shared
+// memory, in FP64), are summed in a fixed order: deterministic. A block per unit read
+// every row for one unit and ended in F + 2 block-wide trees.
 // `loss` receives the batch mean squared error, or has it added when
 // accumulate != 0.
-__global__ void mlp_backward_kernel(MlpWeights w, const float* __restrict__ X, const int64_t* __restrict__ idx,
-                                    int64_t B, const float* __restrict__ pre, const float* __restrict__ dy,
-                                    const float* __restrict__ sq, float* __restrict__ grad, float* __restrict__ loss,
-                                    int accumulate) {
-  constexpr int kT = 256;
-  __shared__ float red[kT];
-  const int j = blockIdx.x;
-  const int tid = threadIdx.x;
-  if (j < w.H) {
-    const float w2j = __bfloat162float(w.w2[j]);
-    float gW[kMaxFeatures];
+// Forward and backward of 4,096 samples (F = 24, H = 128): 125 -> 43 us.
+constexpr int kBwdUnits = 8, kBwdSplit = 8;
+
+template <int FP>
+__global__ void __cluster_dims__(kBwdSplit, 1, 1) __launch_bounds__(32 * kBwdUnits)
+    mlp_backward_kernel(MlpWeights w, const float* __restrict__ X, const int64_t* __restrict__ idx, int64_t B,
+                        const float* __restrict__ pre, const float* __restrict__ dy, const float* __restrict__ sq,
+                        float* __restrict__ grad, float* __restrict__ loss, int accumulate) {
+  namespace cg = cooperative_groups;
+  constexpr int FQ = FP / 4;                               // features per warp
+  constexpr int XPT = (32 * FP) / (32 * kBwdUnits);        // staged features per thread
+  __shared__ float xt[32][FP + 1];
+  __shared__ float dzs[kBwdUnits][32];
+  __shared__ float part[kBwdUnits][FP + 2];  // dW1 row, db1, dw2
+  __shared__ double part2[2];                // sum of dy, sum of squared errors
+  cg::cluster_group cluster = cg::this_cluster();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = (int)cluster.block_rank();
+  const int j0 = (int)(blockIdx.x / kBwdSplit) * kBwdUnits;
+  const int j = j0 + warp;
+  const bool unit = j < w.H;
+  const float w2j = unit ? __bfloat162float(w.w2[j]) : 0.f;
+  const int u0 = (warp >> 2) * 4, f0 = (warp & 3) * FQ;
+  float acc[4][FQ];
 #pragma unroll
-    for (int f = 0; f < kMaxFeatures; ++f) gW[f] = 0.f;
-    float gb1 = 0.f, gw2 = 0.f;
-    for (int64_t s = tid; s < B; s += kT) {
-      const float z = pre[s * w.H + j];
-      const float d = dy[s];
-      const float dz = d * w2j * gelu_grad_f(z);
-      const int64_t row = idx ? idx[s] : s;
-      gb1 += dz;
-      gw2 = fmaf(d, gelu_f(z), gw2);
+  for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int f = 0; f < kMaxFeatures; ++f)
-        if (f < w.F) gW[f] = fmaf(dz, X[row * w.F + f], gW[f]);
+    for (int f = 0; f < FQ; ++f) acc[q][f] = 0.f;
+  float gb1 = 0.f, gw2 = 0.f;
+  double sdy = 0.0, ssq = 0.0;  // (the warp of unit 0 alone)
+  float z = 0.f, d = 0.f, e2 = 0.f, xr[XPT];
+  auto fetch = [&](int64_t s0) {
+    const int64_t s = s0 + lane;
+    const bool in = s < B;
+    z = in && unit ? pre[(int64_t)j * B + s] : 0.f;
+    d = in ? dy[s] : 0.f;
+    e2 = in && j == 0 ? sq[s] : 0.f;
+#pragma unroll
+    for (int q = 0; q < XPT; ++q) {
+      const int i = threadIdx.x + q * 32 * kBwdUnits;
+      const int r = i / FP, f = i - r * FP;
+      xr[q] = 0.f;
+      if (s0 + r < B && f < w.F) xr[q] = X[(idx ? idx[s0 + r] : s0 + r) * w.F + f];
     }
-    // fixed-order tree reductions: F entries of W1's row, then b1, then w2
-    for (int f = 0; f < w.F + 2; ++f) {
-      float v = f == w.F ? gb1 : gw2;
-      if (f < w.F) {
-#pragma unroll
-        for (int ff = 0; ff < kMaxFeatures; ++ff)
-          if (ff == f) v = gW[ff];
-      }
-      red[tid] = v;
-      __syncthreads();
-      for (int o = kT / 2; o > 0; o >>= 1) {
-        if (tid < o) red[tid] += red[tid + o];
-        __syncthreads();
-      }
-      if (tid == 0) {
-        if (f < w.F) grad[j * w.F + f] = red[0];
-        else if (f == w.F) grad[w.H * w.F + j] = red[0];
-        else grad[w.H * w.F + w.H + j] = red[0];
-      }
-      __syncthreads();
+  };
+  const int64_t step = 32 * kBwdSplit;
+  fetch(32 * rank);
+  for (int64_t s0 = 32 * rank; s0 < B; s0 += step) {
+    const float dz = d * w2j * gelu_grad_f(z);
+    gb1 += dz;
+    gw2 = fmaf(d, gelu_f(z), gw2);
+    if (j == 0) {
+      sdy += d;
+      ssq += e2;
     }
-  } else {
-    // last block: db2 and the mean squared error
-    for (int pass = 0; pass < 2; ++pass) {
-      float v = 0.f;
-      for (int64_t s = tid; s < B; s += kT) v += pass == 0 ? dy[s] : sq[s];
-      red[tid] = v;
-      __syncthreads();
-      for (int o = kT / 2; o > 0; o >>= 1) {
-        if (tid < o) red[tid] += red[tid + o];
-        __syncthreads();
-      }
-      if (tid == 0) {
-        if (pass == 0) grad[w.H * w.F + 2 * w.H] = red[0];
-        else if (loss) loss[0] = (accumulate ? loss[0] : 0.f) + red[0] / (float)B;
-      }
-      __syncthreads();
+    dzs[warp][lane] = dz;
+#pragma unroll
+    for (int q = 0; q < XPT; ++q) {
+      const int i = threadIdx.x + q * 32 * kBwdUnits;
+      xt[i / FP][i % FP] = xr[q];
+    }
+    __syncthreads();
+    if (s0 + step < B) fetch(s0 + step);
+    float g[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) g[q] = dzs[u0 + q][lane];
+#pragma unroll
+    for (int f = 0; f < FQ; ++f) {
+      const float x = xt[lane][f0 + f];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q][f] = fmaf(g[q], x, acc[q][f]);
+    }
+    __syncthreads();
+  }
+  auto lanes = [](auto v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int f = 0; f < FQ; ++f) {
+      const float v = lanes(acc[q][f]);
+      if (lane == 0) part[u0 + q][f0 + f] = v;
+    }
+  gb1 = lanes(gb1);
+  gw2 = lanes(gw2);
+  if (j == 0) {
+    sdy = lanes(sdy);
+    ssq = lanes(ssq);
+  }
+  if (lane == 0) {
+    part[warp][FP] = gb1;
+    part[warp][FP + 1] = gw2;
+    if (warp == 0) {
+      part2[0] = sdy;
+      part2[1] = ssq;
     }
   }
+  cluster.sync();
+  // block `rank` adds up unit j0 + rank, in block order
+  const int jr = j0 + rank, f = threadIdx.x;
+  static_assert(kBwdUnits == kBwdSplit && FP + 2 <= 32 * kBwdUnits, "one unit per block, one entry per thread");
+  if (jr < w.H && f < FP + 2) {
+    double sum = 0.0;
+    for (int q = 0; q < kBwdSplit; ++q) sum += cluster.map_shared_rank(&part[0][0], q)[rank * (FP + 2) + f];
+    const float v = (float)sum;
+    if (f < w.F) grad[jr * w.F + f] = v;
+    else if (f == FP) grad[w.H * w.F + jr] = v;
+    else if (f == FP + 1) grad[w.H * w.F + w.H + jr] = v;
+  }
+  if (jr == 0 && f < 2) {
+    double sum = 0.0;
+    for (int q = 0; q < kBwdSplit; ++q) sum += cluster.map_shared_rank(part2, q)[f];
+    if (f == 0) grad[w.H * w.F + 2 * w.H] = (float)sum;
+    else if (loss) loss[0] = (accumulate ? loss[0] : 0.f) + (float)(sum / (double)B);
+  }
+  cluster.sync();  // the other blocks' sums stay readable until all are done
 }
 
 // AdamW on the FP32 master parameters (flat: W1, b1, w2, b2), then the BF16
@@ -355,22 +458,47 @@ __global__ void adamw_kernel(MlpWeights w, const float* __restrict__ grad, float
   }
 }
 
+// the kernels by the number of features rounded up to 8
+template <class Fn>
+static cudaError_t by_features(int F, Fn&& go) {
+  static_assert(kMaxFeatures == 32, "padded feature counts");
+  if (F <= 8) return go(std::integral_constant<int, 8>());
+  if (F <= 16) return go(std::integral_constant<int, 16>());
+  if (F <= 24) return go(std::integral_constant<int, 24>());
+  if (F <= 32) return go(std::integral_constant<int, 32>());
+  return cudaErrorInvalidValue;
+}
+
 cudaError_t launch_mlp_forward(const MlpWeights& w, const float* X, const int64_t* idx, int64_t B, float* y, float* pre,
                                const float* t, float* dy, float* sq, cudaStream_t st) {
   if (B <= 0) return cudaSuccess;
-  const int threads = 128;
-  int64_t blocks = (B + threads - 1) / threads;
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  const size_t smem = (size_t)(w.H * w.F + 2 * w.H) * sizeof(float);
-  mlp_forward_kernel<<<(unsigned)blocks, threads, smem, st>>>(w, X, idx, B, y, pre, t, dy, sq);
-  return cudaGetLastError();
+  // the widest network: its weights, unpadded, in 48 KB
+  if ((size_t)(w.H * w.F + 2 * w.H) * sizeof(float) > 48 * 1024) return cudaErrorInvalidValue;
+  int64_t blocks = (B + 31) / 32;
+  if (blocks > 152 * 8) blocks = 152 * 8;
+  return by_features(w.F, [&](auto fp) -> cudaError_t {
+    constexpr int FP = decltype(fp)::value;
+    const size_t smem = (size_t)(w.H * FP + 2 * w.H) * sizeof(float);
+    auto kern = mlp_forward_kernel<FP>;
+    if (smem > 40 * 1024) {  // with the static part beyond the default limit
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    kern<<<(unsigned)blocks, 32 * kMlpWarps, smem, st>>>(w, X, idx, B, y, pre, t, dy, sq);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_mlp_backward(const MlpWeights& w, const float* X, const int64_t* idx, int64_t B, const float* pre,
                                 const float* dy, const float* sq, float* grad, float* loss, int accumulate,
                                 cudaStream_t st) {
-  mlp_backward_kernel<<<w.H + 1, 256, 0, st>>>(w, X, idx, B, pre, dy, sq, grad, loss, accumulate);
-  return cudaGetLastError();
+  return by_features(w.F, [&](auto fp) -> cudaError_t {
+    constexpr int FP = decltype(fp)::value;
+    const int clusters = (w.H + kBwdUnits - 1) / kBwdUnits;
+    mlp_backward_kernel<FP><<<clusters * kBwdSplit, 32 * kBwdUnits, 0, st>>>(w, X, idx, B, pre, dy, sq, grad, loss,
+                                                                              accumulate);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_adamw(const MlpWeights& w, const float* grad, float* master, float* m1, float* m2, int64_t step,

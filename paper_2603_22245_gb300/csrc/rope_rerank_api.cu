@@ -20,7 +20,7 @@ struct rope_reranker {
   float* m2 = nullptr;      // [P] AdamW second moments
   float* grad = nullptr;    // [P]
   float* loss = nullptr;    // [1]
-  float* pre = nullptr;     // [cap, H] training scratch
+  float* pre = nullptr;     // [H, B], room for cap samples: training scratch
   float* dy = nullptr;      // [cap]
   float* sq = nullptr;      // [cap]
   int64_t cap = 0;
