@@ -647,7 +647,14 @@ rope_status rope::encode_reference_impl(const rope_params* p, const uint8_t* ref
   float2* anchors = nullptr;
   uint16_t *map_lsb = nullptr, *map = nullptr;
   float2 *phase = nullptr, *rot = nullptr, *eout = nullptr, *ein = nullptr;
-  double2 *phase64 = nullptr, *rot64 = nullptr, *eout64 = nullptr, *ein64 = nullptr;
+  double2* phase64 = nullptr;
+  const int n_phase = p->window_len - p->s + 1 + (A - 1) * p->stride;
+  std::vector<double2> chunk_phase((size_t)p->m * n_phase);
+  for (int k = 1; k <= p->m; ++k) {
+    int64_t fa, fq;
+    factor(*p, k, &fa, &fq);
+    for (int d = 0; d < n_phase; ++d) chunk_phase[(size_t)(k - 1) * n_phase + d] = unit(fa, fq, p->window_len, d);
+  }
   if (shared_packed) {
     packed = const_cast<uint32_t*>(shared_packed);  // borrowed: another index owns it
   } else if ((st = upload(idx->owned, std::vector<uint32_t>(), &packed, (size_t)(n_words + pad_words))) != ROPE_OK) {
@@ -665,10 +672,7 @@ rope_status rope::encode_reference_impl(const rope_params* p, const uint8_t* ref
   if ((st = upload(idx->owned, to_f32(h.rot), &rot)) != ROPE_OK) return cleanup(st);
   if ((st = upload(idx->owned, to_f32(h.eout), &eout)) != ROPE_OK) return cleanup(st);
   if ((st = upload(idx->owned, to_f32(h.ein), &ein)) != ROPE_OK) return cleanup(st);
-  if ((st = upload(idx->owned, h.phase, &phase64)) != ROPE_OK) return cleanup(st);
-  if ((st = upload(idx->owned, h.rot, &rot64)) != ROPE_OK) return cleanup(st);
-  if ((st = upload(idx->owned, h.eout, &eout64)) != ROPE_OK) return cleanup(st);
-  if ((st = upload(idx->owned, h.ein, &ein64)) != ROPE_OK) return cleanup(st);
+  if ((st = upload(idx->owned, chunk_phase, &phase64)) != ROPE_OK) return cleanup(st);
 
   DevIndex& ix = idx->ix;
   ix.packed = packed;
@@ -699,8 +703,8 @@ rope_status rope::encode_reference_impl(const rope_params* p, const uint8_t* ref
   cudaError_t e = cudaMemcpy(c->status, &zero, sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && !shared_packed) e = launch_pack(ref, len, packed, c->status, stream);
   if (e == cudaSuccess) {
-    PrepassTables pt{phase64, rot64, eout64, ein64};
-    e = launch_prepass(ix, pt, anchors, inv_norm, band_norm, c->status, stream);
+    const PrepassTables pt{phase64, n_phase};
+    e = launch_prepass(ix, pt, anchors, inv_norm, band_norm, stream);
   }
   if (e != cudaSuccess) return cleanup(fail(ROPE_ERR_CUDA, "index build launch: %s", cudaGetErrorString(e)));
   st = rope_sync_status(stream);

@@ -401,116 +401,195 @@ cudaError_t launch_encode_reads(const EncTables& tb, const uint8_t* seqs, const 
 
 // ---------------------------------------------------------------- reference pre-pass
 
-// One warp per anchor chunk of A windows, in FP64. The chunk's first window is
-// summed directly (§2.1-§2.3); it is stored in FP32 as the anchor that seeds
-// the on-chip FP32 recurrence. The chunk is then walked with the slide
-// relations of §3.4 in FP64 and every window's squared norm (and per-band
-// norms for score_mode 1) is reduced across the warp, so the stored
-// 1/sqrt(C_j) does not inherit the FP32 recurrence's drift.
+// Letters of the packed reference from position p on, one per step: the code of
+// the s letters at the current position, the next word loaded a word ahead.
+struct LetterCursor {
+  const uint32_t* next;
+  uint64_t v;
+  uint32_t ahead;
+  int have;  // letters in v
+  __device__ __forceinline__ void start(const uint32_t* __restrict__ packed, int64_t p) {
+    next = packed + (p >> 4);
+    const int off = (int)(p & 15);
+    v = __ldg(next) >> (2 * off);
+    have = 16 - off;
+    ahead = __ldg(next + 1);
+    next += 2;
+  }
+  __device__ __forceinline__ uint32_t code(int s, uint32_t mask) {
+    if (have < s) {
+      v |= (uint64_t)ahead << (2 * have);
+      have += 16;
+      ahead = __ldg(next++);
+    }
+    const uint32_t c = (uint32_t)v & mask;
+    v >>= 2;
+    --have;
+    return c;
+  }
+};
+
+// 1/sqrt(x) rounded to FP32, x > 0 in FP32's range: an FP32 estimate and one
+// third-order Householder step in FP64 (relative error about e^3 for an
+// estimate's e < 2^-21), 5 FP64 operations where a division and a root take tens.
+__device__ __forceinline__ float inv_sqrt_f64(double x) {
+  const double r = (double)rsqrtf((float)x);
+  const double e = fma(-x * r, r, 1.0);
+  return (float)fma(r * e, fma(0.375, e, 0.5), r);
+}
+
+// Anchors and window norms, in FP64: a lane per (anchor chunk of A windows,
+// band). In the frame of the chunk's first window, w0, a location at offset d
+// adds w_k^d (w_k = e^{2 pi i f_k / N}) to its bin's sum S_{k,b} whatever window
+// it is seen from: window j's entry is S_{k,b} times a unit phase (§3.4's
+// rotation), so norms need no rotation, and sliding by a letter changes
+// C_k = sum_b |S_{k,b}|^2 only through the leaving and the entering bin:
+// |S -+ w|^2 = |S|^2 -+ 2 S.w + 1. A lane keeps its band's sums in shared memory,
+// column = lane (no bank conflicts whatever the bins), sums the first window
+// directly (§2.1-§2.3; stored in FP32, the anchor that seeds the on-chip FP32
+// recurrence) and walks the chunk. The stored 1/sqrt(C_j) thus carries neither
+// the FP32 recurrence's drift nor any rotation's rounding.
+//
+// Bound by the FP64 unit (2 results a cycle per SM): 11 operations a window and
+// band, 2 a location of the first window. A warp per chunk that rotated all D
+// entries and reduced their squares at every window took about 45 FP64
+// instructions of a whole warp a window.
+// Index of 10 Mbp (s = 4, m = t = 2, N = 150), whole call: 38.3 -> 1.74 ms.
+template <bool kUnit>  // stride 1: a window's letters four steps at a time
 __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict__ anchors,
                                float* __restrict__ inv_norm, float* __restrict__ band_norm) {
   extern __shared__ double2 pre_acc[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int wpb = blockDim.x >> 5;
-  double2* acc = pre_acc + (size_t)warp * ix.D;
+  const int m = ix.m, nb = ix.nb, S = ix.stride, s = ix.s;
+  double2* acc = pre_acc + (size_t)warp * nb * 32 + lane;  // entry b: acc[32 * b]
   const int64_t n_chunks = (ix.W + ix.A - 1) / ix.A;
-  const int n_loc = ix.N - ix.s + 1;
-  const int S = ix.stride;
-  for (int64_t a = (int64_t)blockIdx.x * wpb + warp; a < n_chunks; a += (int64_t)gridDim.x * wpb) {
-    const int64_t j0 = a * ix.A;
-    const int64_t w0 = j0 * S;
-    for (int g = lane; g < ix.D; g += 32) acc[g] = make_double2(0.0, 0.0);
-    __syncwarp();
-    for (int loc0 = 0; loc0 < n_loc; loc0 += 32) {
-      const int loc = loc0 + lane;
-      const uint32_t b = loc < n_loc ? bin_at(ix.packed, w0 + loc, ix.s, ix.map_lsb) : 0u;
-      const int cnt = min(32, n_loc - loc0);
-      for (int jj = 0; jj < cnt; ++jj) {
-        const uint32_t bj = __shfl_sync(0xffffffffu, b, jj);
-        if (lane < ix.m) {
-          const double2 ph = pt.phase[lane * n_loc + loc0 + jj];
-          double2& v = acc[lane * ix.nb + bj];
-          v.x += ph.x;
-          v.y += ph.y;
-        }
-        __syncwarp();
+  const int n_loc = ix.N - s + 1;
+  const uint32_t mask = (1u << (2 * s)) - 1u;
+  const int cpw = 32 / m;  // chunks per warp
+  const int k = lane % m;  // this lane's band
+  const int64_t a = ((int64_t)blockIdx.x * wpb + warp) * cpw + lane / m;
+  const bool live = lane < cpw * m && a < n_chunks;
+  // the other lanes walk the last chunk and store nothing
+  const int64_t j0 = (live ? a : n_chunks - 1) * ix.A;
+  const double2* ph = pt.phase + (size_t)k * pt.n_phase;
+  const int group = lane - k;
+
+  for (int b = 0; b < nb; ++b) acc[32 * b] = make_double2(0.0, 0.0);
+  LetterCursor out, in;  // leaving and entering locations
+  out.start(ix.packed, j0 * S);
+  in.start(ix.packed, j0 * S);
+  auto bin = [&](LetterCursor& c) { return (uint32_t)__ldg(ix.map_lsb + c.code(s, mask)); };
+  auto add = [&](uint32_t b, double2 w) {
+    double2 v = acc[32 * b];
+    v.x += w.x;
+    v.y += w.y;
+    acc[32 * b] = v;
+  };
+  {
+    int d = 0;
+    for (; d + 4 <= n_loc; d += 4) {
+      uint32_t b[4];
+      double2 w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        b[q] = bin(in);
+        w[q] = __ldg(ph + d + q);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) add(b[q], w[q]);
+    }
+    for (; d < n_loc; ++d) add(bin(in), __ldg(ph + d));
+  }
+  double C = 0.0;
+  for (int b = 0; b < nb; b += 2) {  // nb = 4^t
+    const double2 v = acc[32 * b], u = acc[32 * (b + 1)];
+    C = fma(v.x, v.x, fma(v.y, v.y, C));
+    C = fma(u.x, u.x, fma(u.y, u.y, C));
+    if (live)
+      *reinterpret_cast<float4*>(anchors + a * ix.D + k * nb + b) = make_float4((float)v.x, (float)v.y, (float)u.x, (float)u.y);
+  }
+  const int n_win = (int)min((int64_t)ix.A, ix.W - j0);
+  // location d leaves for bin bo, location d + n_loc enters bin bi
+  auto slide = [&](uint32_t bo, double2 wo, uint32_t bi, double2 wi) {
+    double2 v = acc[32 * bo];
+    const double p = fma(v.x, wo.x, v.y * wo.y);
+    acc[32 * bo] = make_double2(v.x - wo.x, v.y - wo.y);
+    v = acc[32 * bi];
+    const double q = fma(v.x, wi.x, v.y * wi.y);
+    acc[32 * bi] = make_double2(v.x + wi.x, v.y + wi.y);
+    C = fma(2.0, q - p, C + 2.0);
+  };
+  auto inv_of = [&](int j) -> float {
+    double tot = C;
+    if (m > 1) {
+      tot = 0.0;
+      for (int q = 0; q < m; ++q) tot += __shfl_sync(0xffffffffu, C, (group + q) & 31);
+    }
+    if (band_norm && live && j < n_win) band_norm[(j0 + j) * m + k] = (float)C;
+    return tot > (double)kZeroNorm2 ? inv_sqrt_f64(tot) : 0.f;
+  };
+  for (int jq = 0; jq < kAnchorPeriod; jq += 4) {
+    float inv[4];
+    if (kUnit) {
+      uint32_t bo[4], bi[4];
+      double2 wo[4], wi[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        bo[q] = bin(out);
+        bi[q] = bin(in);
+        // (the slide after the chunk's last window is not needed)
+        const int d = min(jq + q, kAnchorPeriod - 2);
+        wo[q] = __ldg(ph + d);
+        wi[q] = __ldg(ph + d + n_loc);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        inv[q] = inv_of(jq + q);
+        slide(bo[q], wo[q], bi[q], wi[q]);
+      }
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        const float v = inv_of(jq + q);
+        inv[0] = q == 0 ? v : inv[0];
+        inv[1] = q == 1 ? v : inv[1];
+        inv[2] = q == 2 ? v : inv[2];
+        inv[3] = q == 3 ? v : inv[3];
+        if (jq + q == kAnchorPeriod - 1) break;
+        const int d0 = (jq + q) * S;
+        for (int u = 0; u < S; ++u) slide(bin(out), __ldg(ph + d0 + u), bin(in), __ldg(ph + d0 + u + n_loc));
       }
     }
-    // registers: entries g = lane + 32*i
-    double cr[4], ci[4];
-    int kb[4], bb[4];
+    if (live && k == 0) {
+      if (jq + 4 <= n_win) {
+        *reinterpret_cast<float4*>(inv_norm + j0 + jq) = make_float4(inv[0], inv[1], inv[2], inv[3]);
+      } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int g = lane + 32 * i;
-      const bool v = g < ix.D;
-      cr[i] = v ? acc[g].x : 0.0;
-      ci[i] = v ? acc[g].y : 0.0;
-      kb[i] = v ? g / ix.nb : 0;
-      bb[i] = v ? g % ix.nb : -1;
-      if (v) anchors[a * ix.D + g] = make_float2((float)cr[i], (float)ci[i]);
-    }
-    __syncwarp();
-    const int64_t j_end = min(ix.W, j0 + ix.A);
-    for (int64_t j = j0; j < j_end; ++j) {
-      double part = 0.0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) part = fma(cr[i], cr[i], fma(ci[i], ci[i], part));
-      double tot = part;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-      if (lane == 0) inv_norm[j] = tot > (double)kZeroNorm2 ? (float)(1.0 / sqrt(tot)) : 0.f;
-      if (band_norm) {
-        for (int k = 0; k < ix.m; ++k) {
-          double pk = 0.0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (bb[i] >= 0 && kb[i] == k) pk = fma(cr[i], cr[i], fma(ci[i], ci[i], pk));
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) pk += __shfl_xor_sync(0xffffffffu, pk, o);
-          if (lane == 0) band_norm[j * ix.m + k] = (float)pk;
-        }
-      }
-      if (j + 1 < j_end) {
-        const int64_t w = j * S;
-        for (int u = 0; u < S; ++u) {
-          const uint32_t bo = bin_at(ix.packed, w + u, ix.s, ix.map_lsb);
-          const uint32_t bi = bin_at(ix.packed, w + ix.N - ix.s + 1 + u, ix.s, ix.map_lsb);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            if (bb[i] == (int)bo) {
-              const double2 e = pt.eout[kb[i] * S + u];
-              cr[i] -= e.x;
-              ci[i] -= e.y;
-            }
-            if (bb[i] == (int)bi) {
-              const double2 e = pt.ein[kb[i] * S + u];
-              cr[i] += e.x;
-              ci[i] += e.y;
-            }
-          }
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const double2 r = pt.rot[kb[i]];
-          const double xr = cr[i], xi = ci[i];
-          cr[i] = xr * r.x - xi * r.y;
-          ci[i] = xr * r.y + xi * r.x;
-        }
+        for (int q = 0; q < 4; ++q)
+          if (jq + q < n_win) inv_norm[j0 + jq + q] = inv[q];
       }
     }
   }
 }
 
 cudaError_t launch_prepass(const DevIndex& ix, const PrepassTables& pt, float2* anchors, float* inv_norm,
-                           float* band_norm, int* status, cudaStream_t st) {
-  (void)status;
+                           float* band_norm, cudaStream_t st) {
+  static_assert(kAnchorPeriod % 16 == 0, "chunks start at whole packed words and aligned stores of 4 norms");
   const int64_t n_chunks = (ix.W + ix.A - 1) / ix.A;
-  const int wpb = 4;
-  int64_t blocks = (n_chunks + wpb - 1) / wpb;
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  const size_t smem = (size_t)wpb * ix.D * sizeof(double2);
-  prepass_kernel<<<(unsigned)blocks, wpb * 32, smem, st>>>(ix, pt, anchors, inv_norm, band_norm);
+  const int cpw = 32 / ix.m;
+  const int64_t warps = (n_chunks + cpw - 1) / cpw;
+  // 512 nb bytes a warp: 4 warps a block (32 KB at nb = 16), one where the sums
+  // are wide or the reference too short to give every SM a block of 4
+  const int wpb = ix.nb > 16 || warps < 4 * 152 ? 1 : 4;
+  const int64_t blocks = (warps + wpb - 1) / wpb;
+  const size_t smem = (size_t)wpb * ix.nb * 32 * sizeof(double2);
+  if (ix.stride == 1) {
+    prepass_kernel<true><<<(unsigned)blocks, wpb * 32, smem, st>>>(ix, pt, anchors, inv_norm, band_norm);
+  } else {
+    prepass_kernel<false><<<(unsigned)blocks, wpb * 32, smem, st>>>(ix, pt, anchors, inv_norm, band_norm);
+  }
   return cudaGetLastError();
 }
 

@@ -90,13 +90,11 @@ cudaError_t launch_encode_reads(const EncTables& tb, const uint8_t* seqs, const 
 cudaError_t launch_strand_merge(const int64_t* win2, const float* score2, int64_t n, int k, int64_t* out_win,
                                 float* out_score, int8_t* out_strand, cudaStream_t st);
 struct PrepassTables {
-  const double2* phase;  // [m*(N-s+1)]
-  const double2* rot;    // [m]
-  const double2* eout;   // [m*stride]
-  const double2* ein;    // [m*stride]
+  const double2* phase;  // [m * n_phase]: e^{2 pi i f_k d / N} of the locations a chunk's windows reach
+  int32_t n_phase;       // N-s+1 + (kAnchorPeriod-1) * stride
 };
 cudaError_t launch_prepass(const DevIndex& ix, const PrepassTables& pt, float2* anchors, float* inv_norm,
-                           float* band_norm, int* status, cudaStream_t st);
+                           float* band_norm, cudaStream_t st);
 cudaError_t launch_window_embeddings(const DevIndex& ix, int64_t j_begin, int64_t count, float* out,
                                      cudaStream_t st);
 
