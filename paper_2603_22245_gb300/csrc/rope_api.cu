@@ -821,7 +821,7 @@ rope_status plan_scan(const rope_index* idx, int32_t precision, int64_t n_reads,
   ScanPlan pl;
   pl.tc = prec_tc(precision);
   int64_t sup;
-  int group;
+  int group, range_group = 0;
   if (pl.tc) {
     if (!scan_tc_supported(ix.D))
       return fail(ROPE_ERR_UNSUPPORTED, "tensor-core scan built for complex dimension 32 or 64, not %d", ix.D);
@@ -834,7 +834,8 @@ rope_status plan_scan(const rope_index* idx, int32_t precision, int64_t n_reads,
     if (!scan_fp32_supported(ix.D))
       return fail(ROPE_ERR_UNSUPPORTED, "FP32 scan built for complex dimension <= 64, not %d", ix.D);
     sup = scan_fp32_super_tile(ix.D);
-    group = scan_fp32_group(ix.D);
+    group = scan_fp32_group(ix, n_reads);
+    range_group = scan_fp32_range_group();
   } else {
     return fail(ROPE_ERR_INVALID_ARG, "precision %d", precision);
   }
@@ -845,7 +846,9 @@ rope_status plan_scan(const rope_index* idx, int32_t precision, int64_t n_reads,
   a.st0 = (jb / sup) * sup;
   const int64_t n_sup = (je - a.st0 + sup - 1) / sup;
   a.n_groups = (int32_t)((n_reads + group - 1) / group);
-  int64_t nr = n_ranges_req > 0 ? n_ranges_req : (16LL * num_sms + a.n_groups - 1) / a.n_groups;
+  if (range_group == 0) range_group = group;
+  const int64_t n_rg = (n_reads + range_group - 1) / range_group;
+  int64_t nr = n_ranges_req > 0 ? n_ranges_req : (16LL * num_sms + n_rg - 1) / n_rg;
   if (nr < 1) nr = 1;
   if (nr > n_sup) nr = n_sup;
   if (nr > 4096) nr = 4096;
@@ -1253,6 +1256,7 @@ rope_status rope::score_topk_impl(const rope_index* idx, const float* emb_f32, c
     pl.a.norms = norms;
     pl.a.cand_depth = o.cand_depth;
     pl.a.sep = o.sep;
+    pl.a.merge_depth = o.rescore ? o.rescore_depth : o.k;
     pl.a.cand = cand;
     pl.a.dense = nullptr;
     pl.a.status = c->status;
@@ -1663,6 +1667,7 @@ extern "C" rope_status rope_score_topk_noalloc(const rope_index* idx, const floa
     pl.a.norms = norms;
     pl.a.cand_depth = o.cand_depth;
     pl.a.sep = o.sep;
+    pl.a.merge_depth = o.rescore ? o.rescore_depth : o.k;
     pl.a.cand = cand;
     pl.a.dense = nullptr;
     pl.a.status = status;

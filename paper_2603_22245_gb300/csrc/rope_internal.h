@@ -36,6 +36,7 @@ struct ScanArgs {
   int32_t n_groups;
   int32_t cand_depth;        // candidates kept per read per range
   int32_t sep;
+  int32_t merge_depth;       // entries of a read's lists that the merge looks at, best first
   Candidate* cand;           // [n_reads, n_ranges * lists_per_range, cand_depth]
   float* dense;              // [n_reads, je-jb] (dense mode)
   int* status;
@@ -101,7 +102,8 @@ cudaError_t launch_window_embeddings(const DevIndex& ix, int64_t j_begin, int64_
 // rope_scan_fp32.cu
 int scan_fp32_supported(int D);
 int64_t scan_fp32_super_tile(int D);
-int scan_fp32_group(int D);
+int scan_fp32_group(const DevIndex& ix, int64_t n_reads);  // reads per work item
+int scan_fp32_range_group();  // reads per group that the window ranges are laid out for
 cudaError_t launch_scan_fp32(const DevIndex& ix, const ScanArgs& a, bool dense, int num_sms, cudaStream_t st);
 
 // rope_scan_tc.cu

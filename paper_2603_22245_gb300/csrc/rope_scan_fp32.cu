@@ -1,11 +1,21 @@
 // FP32 CUDA-core scan ("plain" path).
 //
-// One thread per read: the read's normalised vector sits in registers; the
+// A thread holds one or two reads' normalised vectors in registers; the
 // block's eight warps generate tiles of window vectors on chip (chains of D/4
 // lanes running the §3.4 recurrence from exact anchors), normalise them by the
 // stored 1/sqrt(C_j) and stage them in shared memory; every thread then forms
 // Re and Im of <x|c> for each window (the §4 real identity) and the fidelity
-// Re^2 + Im^2, keeping its read's best windows in a shared-memory list.
+// Re^2 + Im^2, keeping its reads' best windows in shared-memory lists.
+//
+// Bounds: 4D multiply-adds per read and window on the FP32 units, and the
+// windows' rows as broadcasts from shared memory (a 16-byte load takes four of
+// the SM's 128-byte cycles whether its lanes agree or not): with one read per
+// thread the loads take twice the multiply-adds' time, with two the same. The
+// multiply-adds run as pairs (fma.rn.f32x2 over consecutive entries: the bits of
+// separate sums over even and odd entries), four windows at a time.
+// 500 reads x 2 M windows (d = 64, 8 candidates): 10.4 ms with one read per
+// thread and unbounded lists, 9.7 ms with two, 8.0 ms with bounded lists; what
+// is left beside the multiply-adds is the updates of each list's first windows.
 #include "rope_internal.h"
 #include "rope_topk.cuh"
 
@@ -13,6 +23,23 @@ namespace rope {
 
 constexpr int kF32Threads = 256;  // reads per group
 constexpr int kF32Steps = 8;      // windows per chain per tile
+constexpr int kF32Batch = 4;      // windows scored together
+static_assert(kF32Steps % kF32Batch == 0, "a batch's windows belong to one chain");
+
+constexpr uint64_t kNegPair = 0x8000000080000000ull;  // flips the signs of a pair
+
+// two FP32 values in one 64-bit register, lo in the low half
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+  return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float f32x2_sum(uint64_t v) {
+  return __uint_as_float((uint32_t)v) + __uint_as_float((uint32_t)(v >> 32));
+}
 
 template <int D>
 struct F32Shape {
@@ -24,13 +51,16 @@ struct F32Shape {
   static constexpr size_t kTileBytes = (size_t)TW * 2 * D * sizeof(float);
 };
 
-template <int D, bool kDense, bool kPerBand>
+// R reads per thread: read slots tid and tid + kF32Threads of the group
+template <int D, int R, bool kDense, bool kPerBand>
 __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, ScanArgs a) {
   using Sh = F32Shape<D>;
+  constexpr int kGroup = R * kF32Threads;
+  static_assert(R == 1 || !kPerBand, "per-band scores take one read per thread");
   extern __shared__ __align__(16) uint8_t f32_smem[];
   float* tile = reinterpret_cast<float*>(f32_smem);
   float* list_s = reinterpret_cast<float*>(f32_smem + Sh::kTileBytes);
-  uint32_t* list_w = reinterpret_cast<uint32_t*>(list_s + (size_t)a.cand_depth * kF32Threads);
+  uint32_t* list_w = reinterpret_cast<uint32_t*>(list_s + (size_t)a.cand_depth * kGroup);
 
   const int tid = threadIdx.x;
   const int lane = tid & 31;
@@ -40,46 +70,71 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
   const int S = ix.stride;
   const int n_items = a.n_groups * a.n_ranges;
 
-  ThreadList lst;
-  lst.s = list_s + tid;
-  lst.w = list_w + tid;
-  lst.stride = kF32Threads;
-  lst.depth = a.cand_depth;
+  ThreadList lst[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    lst[i].s = list_s + tid + i * kF32Threads;
+    lst[i].w = list_w + tid + i * kF32Threads;
+    lst[i].stride = kGroup;
+    lst[i].depth = a.cand_depth;
+  }
 
   Chain<D> ch;
   ch.setup(ix, lic);
 
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const int grp = item % a.n_groups;
-    const int rng = item / a.n_groups;
-    const int64_t r = (int64_t)grp * kF32Threads + tid;
+  // items in group-major order, a contiguous run per block: most of a block's
+  // items share their reads
+  const int it_lo = (int)((int64_t)n_items * blockIdx.x / gridDim.x);
+  const int it_hi = (int)((int64_t)n_items * (blockIdx.x + 1) / gridDim.x);
+  // Every range has lists of its own, and a list taking its first windows is
+  // mostly updates. A list that two earlier lists of the read beat with all
+  // their entries cannot add to the merge_depth best of the union, so a window
+  // below the second-largest worst entry of the lists done so far is passed by
+  // (with buckets, sep > 0, entries of two lists may be one: no bound).
+  const bool bounded = !kDense && a.sep == 0 && 2 * a.cand_depth >= a.merge_depth;
+  float first[R], bound[R];  // the two largest worst entries
+  int prev_grp = -1;
+
+  for (int item = it_lo; item < it_hi; ++item) {
+    const int grp = item / a.n_ranges;
+    const int rng = item % a.n_ranges;
+    const int64_t r = (int64_t)grp * kGroup + tid;  // read of slot i: r + i * kF32Threads
     const bool have_read = r < a.n_reads;
     const int64_t st_begin = a.st0 + (int64_t)rng * a.range_len;
     const int64_t j_lo = max(st_begin, a.jb);
     const int64_t j_hi = min(st_begin + a.range_len, a.je);
 
-    // the read's vector, normalised (per band in score mode 1)
-    float xr[D], xi[D];
-    {
-      const float* e = a.emb_f32 + (have_read ? r : 0) * 2 * D;
-      const float* nr = a.norms + (have_read ? r : 0) * (1 + ix.m);
+    // the reads' vectors, normalised (per band in score mode 1)
+    float xr[R][D], xi[R][D];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int64_t ri = r + i * kF32Threads;
+      const bool have = ri < a.n_reads;
+      const float* e = a.emb_f32 + (have ? ri : 0) * 2 * D;
+      const float* nr = a.norms + (have ? ri : 0) * (1 + ix.m);
       float inv = 0.f;
       if (!kPerBand) {
         const float X = nr[0];
-        inv = (have_read && X > kZeroNorm2) ? rsqrtf(X) : 0.f;
+        inv = (have && X > kZeroNorm2) ? rsqrtf(X) : 0.f;
       }
 #pragma unroll
       for (int g = 0; g < D; ++g) {
         float sc = inv;
         if (kPerBand) {
           const float Xk = nr[1 + g / ix.nb];
-          sc = (have_read && Xk > kZeroNorm2) ? rsqrtf(Xk) : 0.f;
+          sc = (have && Xk > kZeroNorm2) ? rsqrtf(Xk) : 0.f;
         }
-        xr[g] = e[g] * sc;
-        xi[g] = e[D + g] * sc;
+        xr[i][g] = e[g] * sc;
+        xi[i][g] = e[D + g] * sc;
+      }
+      if (!kDense) {
+        if (grp != prev_grp) first[i] = bound[i] = -INFINITY;
+        lst[i].reset();
+        lst[i].thr = have ? bound[i] : INFINITY;  // a missing read's list takes nothing
       }
     }
-    if (!kDense) lst.reset();
+
+    prev_grp = grp;
 
     for (int64_t st = st_begin; st < j_hi; st += Sh::SUP) {
       const int64_t a_idx = st / ix.A + chain;
@@ -128,67 +183,91 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
         // ---- score every window of the tile against this thread's read
         if (have_read) {
 #pragma unroll 1
-          for (int q = 0; q < Sh::TW; q += 2) {
-            const float4* c0r = reinterpret_cast<const float4*>(tile + (size_t)q * 2 * D);
-            const float4* c0i = c0r + D / 4;
-            const float4* c1r = c0r + 2 * D / 4;
-            const float4* c1i = c1r + D / 4;
-            float sc0 = 0.f, sc1 = 0.f;
+          for (int q = 0; q < Sh::TW; q += kF32Batch) {
+            float sc[R][kF32Batch];
             if (!kPerBand) {
-              float re0a = 0.f, re0b = 0.f, im0a = 0.f, im0b = 0.f;
-              float re1a = 0.f, re1b = 0.f, im1a = 0.f, im1b = 0.f;
+              // Re and -Im of each window, even and odd entries in the halves of a pair
+              const ulonglong2* c = reinterpret_cast<const ulonglong2*>(tile + (size_t)q * 2 * D);
+              uint64_t re[R][kF32Batch], im[R][kF32Batch];
 #pragma unroll
-              for (int e4 = 0; e4 < D / 4; ++e4) {
-                const float4 ar = c0r[e4], ai = c0i[e4], br = c1r[e4], bi = c1i[e4];
-                const float xa[4] = {xr[4 * e4], xr[4 * e4 + 1], xr[4 * e4 + 2], xr[4 * e4 + 3]};
-                const float ya[4] = {xi[4 * e4], xi[4 * e4 + 1], xi[4 * e4 + 2], xi[4 * e4 + 3]};
-                const float car[4] = {ar.x, ar.y, ar.z, ar.w}, cai[4] = {ai.x, ai.y, ai.z, ai.w};
-                const float cbr[4] = {br.x, br.y, br.z, br.w}, cbi[4] = {bi.x, bi.y, bi.z, bi.w};
+              for (int i = 0; i < R; ++i)
 #pragma unroll
-                for (int h = 0; h < 4; h += 2) {
-                  re0a = fmaf(xa[h], car[h], fmaf(ya[h], cai[h], re0a));
-                  im0a = fmaf(xa[h], cai[h], fmaf(-ya[h], car[h], im0a));
-                  re1a = fmaf(xa[h], cbr[h], fmaf(ya[h], cbi[h], re1a));
-                  im1a = fmaf(xa[h], cbi[h], fmaf(-ya[h], cbr[h], im1a));
-                  re0b = fmaf(xa[h + 1], car[h + 1], fmaf(ya[h + 1], cai[h + 1], re0b));
-                  im0b = fmaf(xa[h + 1], cai[h + 1], fmaf(-ya[h + 1], car[h + 1], im0b));
-                  re1b = fmaf(xa[h + 1], cbr[h + 1], fmaf(ya[h + 1], cbi[h + 1], re1b));
-                  im1b = fmaf(xa[h + 1], cbi[h + 1], fmaf(-ya[h + 1], cbr[h + 1], im1b));
+                for (int h = 0; h < kF32Batch; ++h) re[i][h] = im[i][h] = 0;
+#pragma unroll
+              for (int e4 = 0; e4 < D / 4; ++e4)
+#pragma unroll
+                for (int h = 0; h < kF32Batch; ++h) {
+                  const ulonglong2 cr = c[h * (2 * D / 4) + e4], ci = c[h * (2 * D / 4) + D / 4 + e4];
+                  const uint64_t nx = ci.x ^ kNegPair, ny = ci.y ^ kNegPair;
+#pragma unroll
+                  for (int i = 0; i < R; ++i) {
+                    const uint64_t r0 = f32x2(xr[i][4 * e4], xr[i][4 * e4 + 1]), r1 = f32x2(xr[i][4 * e4 + 2], xr[i][4 * e4 + 3]);
+                    const uint64_t i0 = f32x2(xi[i][4 * e4], xi[i][4 * e4 + 1]), i1 = f32x2(xi[i][4 * e4 + 2], xi[i][4 * e4 + 3]);
+                    re[i][h] = fma_f32x2(r0, cr.x, fma_f32x2(i0, ci.x, re[i][h]));
+                    im[i][h] = fma_f32x2(r0, nx, fma_f32x2(i0, cr.x, im[i][h]));
+                    re[i][h] = fma_f32x2(r1, cr.y, fma_f32x2(i1, ci.y, re[i][h]));
+                    im[i][h] = fma_f32x2(r1, ny, fma_f32x2(i1, cr.y, im[i][h]));
+                  }
                 }
-              }
-              const float re0 = re0a + re0b, im0 = im0a + im0b, re1 = re1a + re1b, im1 = im1a + im1b;
-              sc0 = fmaf(re0, re0, im0 * im0);
-              sc1 = fmaf(re1, re1, im1 * im1);
+#pragma unroll
+              for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int h = 0; h < kF32Batch; ++h) {
+                  const float vr = f32x2_sum(re[i][h]), vi = f32x2_sum(im[i][h]);
+                  sc[i][h] = fmaf(vr, vr, vi * vi);
+                }
             } else {
+#pragma unroll
+              for (int h = 0; h < kF32Batch; ++h) sc[0][h] = 0.f;
               const float* t0 = tile + (size_t)q * 2 * D;
-              const float* t1 = t0 + 2 * D;
               for (int k = 0; k < ix.m; ++k) {
-                float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
+                float re[kF32Batch], im[kF32Batch];
+#pragma unroll
+                for (int h = 0; h < kF32Batch; ++h) re[h] = im[h] = 0.f;
 #pragma unroll
                 for (int g = 0; g < D; ++g) {
                   if (g / ix.nb != k) continue;
-                  re0 = fmaf(xr[g], t0[g], fmaf(xi[g], t0[D + g], re0));
-                  im0 = fmaf(xr[g], t0[D + g], fmaf(-xi[g], t0[g], im0));
-                  re1 = fmaf(xr[g], t1[g], fmaf(xi[g], t1[D + g], re1));
-                  im1 = fmaf(xr[g], t1[D + g], fmaf(-xi[g], t1[g], im1));
-                }
-                sc0 += fmaf(re0, re0, im0 * im0);
-                sc1 += fmaf(re1, re1, im1 * im1);
-              }
-              sc0 /= ix.m;
-              sc1 /= ix.m;
-            }
-            // window numbers of tile slots q, q+1
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int qq = q + h;
-              const int64_t j = st + (int64_t)(qq / kF32Steps) * ix.A + rd * kF32Steps + (qq % kF32Steps);
-              const float sc = h == 0 ? sc0 : sc1;
-              if (j < j_lo || j >= j_hi) continue;
+                  for (int h = 0; h < kF32Batch; ++h) {
+                    const float cr = t0[h * 2 * D + g], ci = t0[h * 2 * D + D + g];
+                    re[h] = fmaf(xr[0][g], cr, fmaf(xi[0][g], ci, re[h]));
+                    im[h] = fmaf(xr[0][g], ci, fmaf(-xi[0][g], cr, im[h]));
+                  }
+                }
+#pragma unroll
+                for (int h = 0; h < kF32Batch; ++h) sc[0][h] += fmaf(re[h], re[h], im[h] * im[h]);
+              }
+#pragma unroll
+              for (int h = 0; h < kF32Batch; ++h) sc[0][h] /= ix.m;
+            }
+            // window numbers of tile slots q .. q+kF32Batch-1 (of one chain)
+            const int64_t jq = st + (int64_t)(q / kF32Steps) * ix.A + rd * kF32Steps + (q % kF32Steps);
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
               if (kDense) {
-                a.dense[r * (a.je - a.jb) + (j - a.jb)] = sc;
-              } else if (sc >= lst.thr) {
-                lst.insert(sc, (uint32_t)j, a.sep, S);
+                const int64_t ri = r + i * kF32Threads;
+                if (ri >= a.n_reads) continue;
+#pragma unroll
+                for (int h = 0; h < kF32Batch; ++h) {
+                  const int64_t j = jq + h;
+                  if (j >= j_lo && j < j_hi) a.dense[ri * (a.je - a.jb) + (j - a.jb)] = sc[i][h];
+                }
+              } else {
+                float top = sc[i][0];
+#pragma unroll
+                for (int h = 1; h < kF32Batch; ++h) top = fmaxf(top, sc[i][h]);
+                if (top < lst[i].thr) continue;
+#pragma unroll 1
+                for (int h = 0; h < kF32Batch; ++h) {
+                  const int64_t j = jq + h;
+                  float v = sc[i][0];
+#pragma unroll
+                  for (int u = 1; u < kF32Batch; ++u) v = h == u ? sc[i][u] : v;
+                  if (j >= j_lo && j < j_hi && v >= lst[i].thr) {
+                    lst[i].insert(v, (uint32_t)j, a.sep, S);
+                    lst[i].thr = fmaxf(lst[i].thr, bound[i]);
+                  }
+                }
               }
             }
           }
@@ -196,9 +275,19 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
         __syncthreads();
       }
     }
-    if (!kDense && have_read) {
-      Candidate* out = a.cand + ((size_t)r * a.n_ranges + rng) * a.cand_depth;
-      for (int e = 0; e < a.cand_depth; ++e) out[e] = Candidate{lst.S(e), lst.Wn(e)};
+    if (!kDense) {
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const int64_t ri = r + i * kF32Threads;
+        if (ri >= a.n_reads) continue;
+        Candidate* out = a.cand + ((size_t)ri * a.n_ranges + rng) * a.cand_depth;
+        for (int e = 0; e < a.cand_depth; ++e) out[e] = Candidate{lst[i].S(e), lst[i].Wn(e)};
+        const float worst = lst[i].S(lst[i].worst);  // -inf: not full
+        if (bounded) {
+          bound[i] = fmaxf(bound[i], fminf(first[i], worst));
+          first[i] = fmaxf(first[i], worst);
+        }
+      }
     }
   }
 }
@@ -216,13 +305,21 @@ int64_t scan_fp32_super_tile(int D) {
   return 0;
 }
 
-int scan_fp32_group(int) { return kF32Threads; }
+// Two reads per thread where one group of 256 does not hold them all: a window
+// read from shared memory then serves twice the multiply-adds (see above). At
+// D = 64 two reads' vectors would not fit in registers.
+static int reads_per_thread(const DevIndex& ix, int64_t n_reads) {
+  return ix.D <= 32 && ix.score_mode == 0 && n_reads > kF32Threads ? 2 : 1;
+}
 
-template <int D, bool kDense, bool kPerBand>
+int scan_fp32_group(const DevIndex& ix, int64_t n_reads) { return kF32Threads * reads_per_thread(ix, n_reads); }
+int scan_fp32_range_group() { return kF32Threads; }
+
+template <int D, int R, bool kDense, bool kPerBand>
 static cudaError_t launch_one(const DevIndex& ix, const ScanArgs& a, int num_sms, cudaStream_t st) {
   using Sh = F32Shape<D>;
-  const size_t smem = Sh::kTileBytes + (kDense ? 0 : (size_t)a.cand_depth * kF32Threads * 8);
-  auto kern = scan_fp32_kernel<D, kDense, kPerBand>;
+  const size_t smem = Sh::kTileBytes + (kDense ? 0 : (size_t)a.cand_depth * kF32Threads * R * 8);
+  auto kern = scan_fp32_kernel<D, R, kDense, kPerBand>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
@@ -237,14 +334,22 @@ static cudaError_t launch_one(const DevIndex& ix, const ScanArgs& a, int num_sms
   return cudaGetLastError();
 }
 
+template <int D, bool kDense, bool kPerBand>
+static cudaError_t by_reads(const DevIndex& ix, const ScanArgs& a, int num_sms, cudaStream_t st) {
+  if constexpr (D <= 32 && !kPerBand) {
+    if (reads_per_thread(ix, a.n_reads) == 2) return launch_one<D, 2, kDense, kPerBand>(ix, a, num_sms, st);
+  }
+  return launch_one<D, 1, kDense, kPerBand>(ix, a, num_sms, st);
+}
+
 template <bool kDense, bool kPerBand>
 static cudaError_t dispatch(const DevIndex& ix, const ScanArgs& a, int num_sms, cudaStream_t st) {
   switch (ix.D) {
-    case 4: return launch_one<4, kDense, kPerBand>(ix, a, num_sms, st);
-    case 8: return launch_one<8, kDense, kPerBand>(ix, a, num_sms, st);
-    case 16: return launch_one<16, kDense, kPerBand>(ix, a, num_sms, st);
-    case 32: return launch_one<32, kDense, kPerBand>(ix, a, num_sms, st);
-    case 64: return launch_one<64, kDense, kPerBand>(ix, a, num_sms, st);
+    case 4: return by_reads<4, kDense, kPerBand>(ix, a, num_sms, st);
+    case 8: return by_reads<8, kDense, kPerBand>(ix, a, num_sms, st);
+    case 16: return by_reads<16, kDense, kPerBand>(ix, a, num_sms, st);
+    case 32: return by_reads<32, kDense, kPerBand>(ix, a, num_sms, st);
+    case 64: return by_reads<64, kDense, kPerBand>(ix, a, num_sms, st);
   }
   return cudaErrorInvalidValue;
 }
