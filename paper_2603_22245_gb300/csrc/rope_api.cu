@@ -1582,11 +1582,9 @@ extern "C" rope_status rope_map_strands(const rope_index* idx, const uint8_t* se
   float* score2 = reinterpret_cast<float*>(scratch + b_f32 + b_norm + b_win);
   uint16_t* embh = reinterpret_cast<uint16_t*>(scratch + b_f32 + b_norm + b_win + b_sc);
   const int slot = prof_begin(stream);
-  cudaError_t e = launch_encode_reads(idx->enc, seqs, offsets, n_reads, emb, embh, norms, c->status, stream);
-  if (e == cudaSuccess)
-    e = launch_encode_reads(idx->enc, seqs, offsets, n_reads, emb + (size_t)n_reads * 2 * D,
-                            embh + (size_t)n_reads * 2 * D, norms + (size_t)n_reads * (1 + m), c->status, stream,
-                            nullptr, true);
+  // (both strands in one launch)
+  cudaError_t e = launch_encode_reads(idx->enc, seqs, offsets, n_reads, emb, embh, norms, c->status, stream, nullptr,
+                                      n_reads);
   prof_mark(slot, 1, stream);
   if (e != cudaSuccess) st = fail(ROPE_ERR_CUDA, "encode launch: %s", cudaGetErrorString(e));
   if (st == ROPE_OK) {

@@ -134,7 +134,7 @@ constexpr int kEncMaxBinBits = 8;  // bins per band up to 256
 __global__ void encode_reads_kernel(EncTables tb, const uint8_t* __restrict__ seqs,
                                     const int64_t* __restrict__ offsets, int64_t n, float* __restrict__ emb_f32,
                                     __nv_bfloat16* __restrict__ emb_bf16, float* __restrict__ norms, int* status,
-                                    const int64_t* __restrict__ perm, bool rc) {
+                                    const int64_t* __restrict__ perm, int64_t n_fwd) {
   extern __shared__ float2 enc_phase[];  // [m * n_loc] phases, staged once per block
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -152,7 +152,8 @@ __global__ void encode_reads_kernel(EncTables tb, const uint8_t* __restrict__ se
     bin[e] = g < tb.D ? g % tb.nb : -1;  // -1: no entry
   }
   for (int64_t r = (int64_t)blockIdx.x * wpb + warp; r < n; r += (int64_t)gridDim.x * wpb) {
-    const int64_t src = perm ? perm[r] : r;
+    const bool rc = r >= n_fwd;
+    const int64_t src = rc ? r - n_fwd : perm ? perm[r] : r;
     const int64_t start = offsets[src];
     const int64_t len = offsets[src + 1] - start;
     const uint8_t* seq = seqs + start;
@@ -244,13 +245,15 @@ __global__ void encode_reads_kernel(EncTables tb, const uint8_t* __restrict__ se
 // §2.1-§2.3 direct sum). The phases of kEncChunk locations are staged in
 // shared memory once per block for all of its warps.
 // A step of 32 locations is a chain (letters, s-mer codes, the bin table, which
-// at 4^8 codes lies in L2, the group's sum), so letters are loaded two steps and
+// at 4^8 codes lies in L2, the group's sum), so letters are loaded three steps and
 // bins one step ahead, codes come from bit planes of the letters, and only the
 // groups' lowest lanes walk their group.
 // 2,048 heads of 20,000 letters on both strands (s = 8, 4 bands of 256 bins)
 // mapped against 30 Mbp, whole call: 3.75 ms with every lane following the
-// largest group by shuffles and nothing loaded ahead, now 2.49 ms.
-constexpr int kEncChunk = 1024;
+// largest group by shuffles and nothing loaded ahead, 2.49 ms so, and 1.89 ms
+// with both strands in one launch and a block per SM that holds all of its heads.
+constexpr int kEncChunk = 256;
+constexpr int kEncWideWarps = 28;  // most warps of a block (72 registers a thread)
 
 // bit i of v (i < 8) at bit 2i
 __device__ __forceinline__ uint32_t spread_bits(uint32_t v) {
@@ -259,10 +262,10 @@ __device__ __forceinline__ uint32_t spread_bits(uint32_t v) {
   return (v | (v << 1)) & 0x5555u;
 }
 
-__global__ void encode_reads_wide_kernel(EncTables tb, const uint8_t* __restrict__ seqs,
+__global__ void __launch_bounds__(32 * kEncWideWarps) encode_reads_wide_kernel(EncTables tb, const uint8_t* __restrict__ seqs,
                                     const int64_t* __restrict__ offsets, int64_t n, float* __restrict__ emb_f32,
                                     __nv_bfloat16* __restrict__ emb_bf16, float* __restrict__ norms, int* status,
-                                    const int64_t* __restrict__ perm, bool rc) {
+                                    const int64_t* __restrict__ perm, int64_t n_fwd) {
   extern __shared__ float2 enc_sm[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -273,7 +276,8 @@ __global__ void encode_reads_wide_kernel(EncTables tb, const uint8_t* __restrict
   for (int64_t r0 = (int64_t)blockIdx.x * wpb; r0 < n; r0 += (int64_t)gridDim.x * wpb) {
     const int64_t r = r0 + warp;
     const bool live = r < n;
-    const int64_t src = live ? (perm ? perm[r] : r) : 0;
+    const bool rc = live && r >= n_fwd;
+    const int64_t src = !live ? 0 : rc ? r - n_fwd : perm ? perm[r] : r;
     const int64_t start = live ? offsets[src] : 0;
     const int64_t len = live ? offsets[src + 1] - start : 0;
     const uint8_t* seq = seqs + start;
@@ -288,11 +292,13 @@ __global__ void encode_reads_wide_kernel(EncTables tb, const uint8_t* __restrict
     bad |= ahead;
     uint32_t lo0 = __ballot_sync(0xffffffffu, ahead & 1u), lo1 = __ballot_sync(0xffffffffu, ahead & 2u);
     ahead = letter(32 + lane);
+    uint32_t ahead2 = letter(64 + lane);
     // bin of location l0 + lane, called for l0 = 0, 32, ...
     auto next_bin = [&](int l0) -> uint32_t {
       bad |= ahead;
       const uint32_t hi0 = __ballot_sync(0xffffffffu, ahead & 1u), hi1 = __ballot_sync(0xffffffffu, ahead & 2u);
-      ahead = letter(l0 + 64 + lane);
+      ahead = ahead2;
+      ahead2 = letter(l0 + 96 + lane);
       const uint32_t code = (spread_bits(__brev(__funnelshift_r(lo0, hi0, lane)) >> (32 - tb.s))) |
                             (spread_bits(__brev(__funnelshift_r(lo1, hi1, lane)) >> (32 - tb.s)) << 1);
       lo0 = hi0;
@@ -380,8 +386,10 @@ __global__ void encode_reads_wide_kernel(EncTables tb, const uint8_t* __restrict
 
 cudaError_t launch_encode_reads(const EncTables& tb, const uint8_t* seqs, const int64_t* offsets, int64_t n,
                                 float* emb_f32, uint16_t* emb_bf16, float* norms, int* status, cudaStream_t st,
-                                const int64_t* perm, bool rc) {
+                                const int64_t* perm, int64_t n_rc) {
   if (n <= 0) return cudaSuccess;
+  const int64_t n_fwd = n;
+  n += n_rc;
   const size_t phase_bytes = (size_t)tb.m * (tb.N - tb.s + 1) * sizeof(float2);
   if (tb.D <= kMaxScanDim && phase_bytes <= 48 * 1024) {
     const int wpb = 8;
@@ -389,20 +397,26 @@ cudaError_t launch_encode_reads(const EncTables& tb, const uint8_t* seqs, const 
     if (blocks > 152 * 16) blocks = 152 * 16;  // each block stages the phase table once
     encode_reads_kernel<<<(unsigned)blocks, wpb * 32, phase_bytes, st>>>(tb, seqs, offsets, n, emb_f32,
                                                                  reinterpret_cast<__nv_bfloat16*>(emb_bf16), norms,
-                                                                 status, perm, rc);
+                                                                 status, perm, n_fwd);
     return cudaGetLastError();
   }
-  // phase chunk + one accumulator per warp, within 100 KB (two blocks per SM)
+  // A step is latency, so an SM wants as many heads at a time as it is going to
+  // get: one block per SM with a warp for each of the SM's heads, or, where their
+  // sums do not fit in its shared memory, an equal share in each wave.
+  int dev = 0, sms = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
   const size_t chunk_bytes = (size_t)tb.m * kEncChunk * sizeof(float2);
-  int wpb = (int)((100 * 1024 - chunk_bytes) / (tb.D * sizeof(float2)));
-  if (wpb > 8) wpb = 8;
-  if (wpb < 1) wpb = 1;
+  int64_t most = ((size_t)optin - chunk_bytes) / (tb.D * sizeof(float2));
+  if (most > kEncWideWarps) most = kEncWideWarps;
+  if (most < 1) most = 1;
+  const int64_t waves = (n + sms * most - 1) / (sms * most);
+  const int wpb = (int)((n + sms * waves - 1) / (sms * waves));
   const size_t smem = chunk_bytes + (size_t)wpb * tb.D * sizeof(float2);
   static int attr_set[64] = {};  // per device: bytes the attribute was last raised to
-  int dev = 0;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || (int)smem > attr_set[dev]) {
       e = cudaFuncSetAttribute(encode_reads_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
@@ -413,7 +427,7 @@ cudaError_t launch_encode_reads(const EncTables& tb, const uint8_t* seqs, const 
   if (blocks > 152 * 16) blocks = 152 * 16;
   encode_reads_wide_kernel<<<(unsigned)blocks, wpb * 32, smem, st>>>(tb, seqs, offsets, n, emb_f32,
                                                                        reinterpret_cast<__nv_bfloat16*>(emb_bf16),
-                                                                       norms, status, perm, rc);
+                                                                       norms, status, perm, n_fwd);
   return cudaGetLastError();
 }
 
