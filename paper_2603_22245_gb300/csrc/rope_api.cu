@@ -257,7 +257,7 @@ rope_status upload(std::vector<void*>& owned, const std::vector<T>& v, T** out) 
 // its padding. Kernels write every element of an array, so only the padding is
 // cleared. A cudaMalloc, a cudaMemset and a cudaMemcpy for each of a dozen parts,
 // and a cudaFree for each at the end, took longer than the build's kernels.
-// Index of 10 Mbp: 1.74 -> 1.49 ms (d = 64), 2.67 -> 2.42 ms (materialised, D = 1,024).
+// Index of 10 Mbp: 1.74 -> 1.50 ms (d = 64), 2.67 -> 2.42 ms (materialised, D = 1,024).
 class IndexBlock {
  public:
   template <class T>

@@ -486,7 +486,8 @@ __device__ __forceinline__ float inv_sqrt_f64(double x) {
 // band, 2 a location of the first window. A warp per chunk that rotated all D
 // entries and reduced their squares at every window took about 45 FP64
 // instructions of a whole warp a window.
-// Index of 10 Mbp (s = 4, m = t = 2, N = 150), whole call: 38.3 -> 1.74 ms.
+// Index of 10 Mbp (s = 4, m = t = 2, N = 150), whole call: 38.3 -> 1.74 ms, and
+// 1.50 -> 1.31 ms by forming each root once instead of in every band's lane.
 template <bool kUnit>  // stride 1: a window's letters four steps at a time
 __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict__ anchors,
                                float* __restrict__ inv_norm, float* __restrict__ band_norm) {
@@ -553,17 +554,18 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
     acc[32 * bi] = make_double2(v.x + wi.x, v.y + wi.y);
     C = fma(2.0, q - p, C + 2.0);
   };
-  auto inv_of = [&](int j) -> float {
+  // C of window j over all bands
+  auto total_of = [&](int j) -> double {
     double tot = C;
     if (m > 1) {
       tot = 0.0;
       for (int q = 0; q < m; ++q) tot += __shfl_sync(0xffffffffu, C, (group + q) & 31);
     }
     if (band_norm && live && j < n_win) band_norm[(j0 + j) * m + k] = (float)C;
-    return tot > (double)kZeroNorm2 ? inv_sqrt_f64(tot) : 0.f;
+    return tot;
   };
   for (int jq = 0; jq < kAnchorPeriod; jq += 4) {
-    float inv[4];
+    double tot[4];
     if (kUnit) {
       uint32_t bo[4], bi[4];
       double2 wo[4], wi[4];
@@ -578,37 +580,33 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        inv[q] = inv_of(jq + q);
+        tot[q] = total_of(jq + q);
         slide(bo[q], wo[q], bi[q], wi[q]);
       }
     } else {
 #pragma unroll 1
       for (int q = 0; q < 4; ++q) {
-        const float v = inv_of(jq + q);
-        inv[0] = q == 0 ? v : inv[0];
-        inv[1] = q == 1 ? v : inv[1];
-        inv[2] = q == 2 ? v : inv[2];
-        inv[3] = q == 3 ? v : inv[3];
+        const double v = total_of(jq + q);
+        tot[0] = q == 0 ? v : tot[0];
+        tot[1] = q == 1 ? v : tot[1];
+        tot[2] = q == 2 ? v : tot[2];
+        tot[3] = q == 3 ? v : tot[3];
         if (jq + q == kAnchorPeriod - 1) break;
         const int d0 = (jq + q) * S;
         for (int u = 0; u < S; ++u) slide(bin(out), __ldg(ph + d0 + u), bin(in), __ldg(ph + d0 + u + n_loc));
       }
     }
-    if (live && k == 0) {
-      if (jq + 4 <= n_win) {
-        *reinterpret_cast<float4*>(inv_norm + j0 + jq) = make_float4(inv[0], inv[1], inv[2], inv[3]);
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (jq + q < n_win) inv_norm[j0 + jq + q] = inv[q];
-      }
+    // the four roots are shared among the chunk's lanes (each knows all totals)
+    for (int q = k; q < 4; q += m) {
+      const double v = q < 2 ? (q == 0 ? tot[0] : tot[1]) : (q == 2 ? tot[2] : tot[3]);
+      if (live && jq + q < n_win) inv_norm[j0 + jq + q] = v > (double)kZeroNorm2 ? inv_sqrt_f64(v) : 0.f;
     }
   }
 }
 
 cudaError_t launch_prepass(const DevIndex& ix, const PrepassTables& pt, float2* anchors, float* inv_norm,
                            float* band_norm, cudaStream_t st) {
-  static_assert(kAnchorPeriod % 16 == 0, "chunks start at whole packed words and aligned stores of 4 norms");
+  static_assert(kAnchorPeriod % 16 == 0, "chunks start at whole packed words; windows go four at a time");
   const int64_t n_chunks = (ix.W + ix.A - 1) / ix.A;
   const int cpw = 32 / ix.m;
   const int64_t warps = (n_chunks + cpw - 1) / cpw;
