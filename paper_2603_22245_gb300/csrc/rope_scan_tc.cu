@@ -103,6 +103,7 @@ struct TcShape {
   static constexpr int TMEM_COLS = 512;
   static constexpr int NACC = TMEM_COLS / (2 * T);     // accumulators of one (stage, read tile) each
   static constexpr int STG = NACC / NT;                // accumulators per read tile, used in turn
+  static constexpr int STEP = NM / NT;                 // MMA issuers a tile's stages alternate over
   static constexpr int BIN_PITCH = A + 4;              // stride 1: bytes of one chain's row of bins
   static constexpr uint32_t IDESC = FP8 ? idesc_e4m3_f32(128, 2 * T) : idesc_bf16_f32(128, 2 * T);
   static constexpr float SCORE_SCALE = FP8 ? 1.f / (kFp8Scale * kFp8Scale * kFp8Scale * kFp8Scale) : 1.f;
@@ -117,6 +118,7 @@ struct TcShape {
   static_assert(D == 32 || D == 64, "complex dimension");
   static_assert(GEN_WARPS * CPW == T, "T must be a multiple of chains per warp");
   static_assert((NM == 2 || NM == 4) && NM % NT == 0 && (NM == NT || NM == NT * STG) && STG >= 1 && STG * NT * 2 * T <= TMEM_COLS, "tensor memory budget");
+  static_assert(A % STEP == 0, "every item starts at the first of a tile's issuers");
   static_assert(WPH % 16 == 0 && LPW >= 1 && (LPW == 1 || WPH % (16 * LPW) == 0), "the epilogue loads 16-column chunks");
   static_assert(BPL * EB == 8 || (BPL * EB) % 16 == 0, "generator lanes write 8-byte or whole 16-byte pieces");
   static_assert(KBLK == 64 || KBLK == 128, "swizzle row");
@@ -621,8 +623,15 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
     // (k NT + t) mod NM = x. A single thread's path through a unit (two barrier
     // waits, the MMAs, two commits) is longer than the tensor pipe's time for
     // it; with several in turn the pipe does not wait for it.
+    //
+    // A wait names a fill of a slot by its parity alone, so a thread may wait for
+    // a stage only once the slot's previous fill is complete. A thread that waits
+    // for stage k has seen stage k - STEP filled, and with it (generators fill in
+    // order) every earlier one: the slot's previous fill, stage k - nb, is among
+    // them if nb >= STEP. The launch takes a shape with one issuer per tile where
+    // shared memory leaves fewer slots.
     if (lane == 0) {
-      constexpr int NM = Sh::NM, STEP = NM / NT;  // a thread's units lie in every STEP-th stage
+      constexpr int STEP = Sh::STEP;  // a thread's units lie in every STEP-th stage
       const int x = Sh::mma_index(warp);
       const int t = x % NT;
       uint32_t it = 0, use = 0;
@@ -1004,17 +1013,26 @@ static size_t tc_smem_bytes(const DevIndex& ix, int cand_depth, bool lists, int 
          (size_t)n_bin * L.bins_bytes + list_bytes;
 }
 
+// The same tiles with one MMA issuer per read tile, for a ring of one slot.
+template <class Sh>
+using TcOneSlot = TcShape<Sh::D, Sh::NT, Sh::T, 1, Sh::LPC, Sh::EW, Sh::LH, Sh::NT, Sh::ISOLATE_MMA, Sh::FP8>;
+
 // The most B slots, with two buffers of bins before one and whole queues before
-// queues of one entry, that fit in `limit` bytes; 0 if none do.
+// shorter ones, that fit in `limit` bytes; 0 if none do. Where a tile has two MMA
+// issuers, two slots with a shorter queue come before one slot.
 template <class Sh>
 static size_t tc_plan_smem(const DevIndex& ix, int cand_depth, bool lists, size_t limit, TcLaunch* L) {
   for (int n_bin = 2; n_bin >= 1; --n_bin)
-    for (int nb = Sh::NB; nb >= (n_bin == 2 ? 2 : 1); --nb) {
+    for (int nb = Sh::NB; nb >= 2; --nb) {
       const size_t b = tc_smem_bytes<Sh>(ix, cand_depth, lists, nb, n_bin, kPend, L);
       if (b <= limit) return b;
     }
-  const size_t b = tc_smem_bytes<Sh>(ix, cand_depth, lists, 1, 1, 1, L);
-  return b <= limit ? b : 0;
+  for (int nb = Sh::STEP; nb >= 1; --nb)
+    for (int pend = kPend; pend >= 1; --pend) {
+      const size_t b = tc_smem_bytes<Sh>(ix, cand_depth, lists, nb, 1, pend, L);
+      if (b <= limit) return b;
+    }
+  return 0;
 }
 
 // Whether the scan takes candidate lists of this depth: tiles, lists and one B
@@ -1049,6 +1067,13 @@ static cudaError_t launch_tc(const DevIndex& ix, const ScanArgs& a, int num_sms,
   TcLaunch L;
   const size_t smem = tc_plan_smem<Sh>(ix, a.cand_depth, !(kDense || kThr), tc_dyn_limit<Sh, kDense, kThr>(), &L);
   if (smem == 0) return cudaErrorInvalidValue;
+  if constexpr (Sh::STEP > 1) {
+    if (L.nb < Sh::STEP) {
+      // (without lists two slots always fit: 214 KB at the longest windows and the largest stride)
+      if constexpr (kDense || kThr) return cudaErrorInvalidValue;
+      else return launch_tc<TcOneSlot<Sh>, kDense, kThr>(ix, a, num_sms, st, thr);
+    }
+  }
   L.thr = thr ? *thr : ThrOut{};
   auto kern = scan_tc_kernel<Sh, kDense, kThr>;
   cudaError_t e = tc_reserve_smem<Sh, kDense, kThr>(smem);
