@@ -97,6 +97,30 @@ extern "C" rope_status rope_set_wait_limit(double seconds) {
   return ROPE_OK;
 }
 
+cudaError_t rope::allow_smem(const void* kern, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::pair<int, const void*>, size_t> most;  // (device, kernel): the limit it was given
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  auto it = most.find({dev, kern});
+  if (it == most.end()) {
+    int optin = 0;
+    cudaFuncAttributes fa{};
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+    const size_t room = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // not sticky: leave no pending error for later launches
+      return e;
+    }
+    it = most.emplace(std::make_pair(dev, kern), room).first;
+  }
+  return smem <= it->second ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // ---------------------------------------------------------------- per-device context
 
 namespace {

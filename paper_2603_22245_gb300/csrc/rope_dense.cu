@@ -205,24 +205,20 @@ cudaError_t launch_dense_index(const DevIndex& ix, const DenseTables& dt, float2
     int wpb = (int)((96 * 1024) / ((size_t)ix.D * sizeof(float2)));  // accumulators within 96 KB
     wpb = wpb < 1 ? 1 : wpb > 8 ? 8 : wpb;
     const size_t smem = (size_t)wpb * ix.D * sizeof(float2);
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(block_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = allow_smem(block_sums_kernel, smem);
+    if (e != cudaSuccess) return e;
     int64_t blocks = (dt.n_blocks + wpb - 1) / wpb;
     if (blocks > 152 * 32) blocks = 152 * 32;
     block_sums_kernel<<<(unsigned)blocks, wpb * 32, smem, st>>>(ix, dt, bsum);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   const int64_t run = 32;
   const int64_t grid = (ix.W + run - 1) / run;
   const size_t smem = (size_t)ix.D * sizeof(float2);
   auto go = [&](auto kern) -> cudaError_t {
-    if (smem > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<(unsigned)grid, 256, smem, st>>>(ix, dt, bsum, win_f32, reinterpret_cast<__nv_bfloat16*>(win_bf16),
                                             reinterpret_cast<__nv_bfloat16*>(win_bf16_im), inv_norm, run);
     return cudaGetLastError();
@@ -751,8 +747,7 @@ cudaError_t launch_dense_fp32(const DevIndex& ix, const GemmArgs& g, const float
   const size_t smem = (size_t)g.cand_depth * kF32Tile * 8;
   // lists of up to 32 entries (16 KB) beside 33 KB of static tiles: past the
   // default 48 KB per block
-  const cudaError_t attr =
-      cudaFuncSetAttribute(dense_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t attr = allow_smem(dense_fp32_kernel, smem);
   if (attr != cudaSuccess) return attr;
   dense_fp32_kernel<<<(unsigned)grid, 256, smem, st>>>(ix, g, emb, norms);
   return cudaGetLastError();
@@ -790,11 +785,8 @@ cudaError_t launch_gemm_tc(const CUtensorMap& tmA, const CUtensorMap& tmB, const
   const size_t smem = short_k ? GemmShape<true>::smem_bytes(g.stages, mode == 0 ? g.cand_depth : 0, g.k_blocks)
                               : GemmShape<false>::smem_bytes(g.stages, mode == 0 ? g.cand_depth : 0, g.k_blocks);
   auto go = [&](auto kern, int threads) -> cudaError_t {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e;
-    }
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<grid, threads, smem, st>>>(tmA, tmB, tmBi, g);
     return cudaGetLastError();
   };

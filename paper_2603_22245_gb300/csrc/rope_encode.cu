@@ -423,14 +423,8 @@ cudaError_t launch_encode_reads(const EncTables& tb, const uint8_t* seqs, const 
   const int64_t waves = (n + sms * most - 1) / (sms * most);
   const int wpb = (int)((n + sms * waves - 1) / (sms * waves));
   const size_t smem = chunk_bytes + (size_t)wpb * tb.D * sizeof(float2);
-  static int attr_set[64] = {};  // per device: bytes the attribute was last raised to
-  if (smem > 48 * 1024) {
-    if (dev < 0 || dev >= 64 || (int)smem > attr_set[dev]) {
-      e = cudaFuncSetAttribute(encode_reads_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) attr_set[dev] = (int)smem;
-    }
-  }
+  e = allow_smem(encode_reads_wide_kernel, smem);
+  if (e != cudaSuccess) return e;
   int64_t blocks = (n + wpb - 1) / wpb;
   if (blocks > 152 * 16) blocks = 152 * 16;
   encode_reads_wide_kernel<<<(unsigned)blocks, wpb * 32, smem, st>>>(tb, seqs, offsets, n, emb_f32,

@@ -11,6 +11,17 @@
 
 namespace rope {
 
+// Lets launches of `kern` on the current device take `smem` bytes of dynamic
+// shared memory (cudaErrorInvalidValue if a block cannot). Setting a kernel's
+// limit replaces it for every thread of the process, so a limit that followed each
+// launch's size could be lowered between another thread's setting and its launch:
+// it is set once per device, to the most a block of the kernel can take.
+cudaError_t allow_smem(const void* kern, size_t smem);
+template <class... A>
+cudaError_t allow_smem(void (*kern)(A...), size_t smem) {
+  return allow_smem(reinterpret_cast<const void*>(kern), smem);
+}
+
 // Tables a read encoder needs (device pointers).
 struct EncTables {
   int32_t N, s, m, t, nb, D;

@@ -455,7 +455,7 @@ static int ceil_log2(int64_t v) {
 template <int MB>
 static cudaError_t launch_bands(RefineArgs a, int warps, size_t smem, int num_sms, cudaStream_t st) {
   auto kern = refine_kernel<MB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, warps * 32, smem);

@@ -480,10 +480,8 @@ cudaError_t launch_mlp_forward(const MlpWeights& w, const float* X, const int64_
     constexpr int FP = decltype(fp)::value;
     const size_t smem = (size_t)(w.H * FP + 2 * w.H) * sizeof(float);
     auto kern = mlp_forward_kernel<FP>;
-    if (smem > 40 * 1024) {  // with the static part beyond the default limit
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     kern<<<(unsigned)blocks, 32 * kMlpWarps, smem, st>>>(w, X, idx, B, y, pre, t, dy, sq);
     return cudaGetLastError();
   });

@@ -320,7 +320,7 @@ static cudaError_t launch_one(const DevIndex& ix, const ScanArgs& a, int num_sms
   using Sh = F32Shape<D>;
   const size_t smem = Sh::kTileBytes + (kDense ? 0 : (size_t)a.cand_depth * kF32Threads * R * 8);
   auto kern = scan_fp32_kernel<D, R, kDense, kPerBand>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kern, smem);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kF32Threads, smem);

@@ -954,20 +954,6 @@ static size_t tc_dyn_limit() {
   return v;
 }
 
-// Raises the kernel's dynamic shared-memory limit on the current device when
-// a launch needs more than it was last set to (once per size increase).
-template <class Sh, bool kDense, bool kThr = false>
-static cudaError_t tc_reserve_smem(size_t smem) {
-  static size_t set[kMaxDevices] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < kMaxDevices && set[dev] >= smem) return cudaSuccess;
-  e = cudaFuncSetAttribute(scan_tc_kernel<Sh, kDense, kThr>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && dev >= 0 && dev < kMaxDevices) set[dev] = smem;
-  return e;
-}
-
 int scan_tc_supported(int D) { return D == 32 || D == 64; }
 
 int64_t scan_tc_super_tile(int D, int variant) {
@@ -1076,11 +1062,8 @@ static cudaError_t launch_tc(const DevIndex& ix, const ScanArgs& a, int num_sms,
   }
   L.thr = thr ? *thr : ThrOut{};
   auto kern = scan_tc_kernel<Sh, kDense, kThr>;
-  cudaError_t e = tc_reserve_smem<Sh, kDense, kThr>(smem);
-  if (e != cudaSuccess) {
-    cudaGetLastError();  // not sticky: leave no pending error for later launches
-    return e;
-  }
+  const cudaError_t e = allow_smem(kern, smem);
+  if (e != cudaSuccess) return e;
   const int64_t n_items = (int64_t)a.n_groups * a.n_ranges;
   const int grid = (int)(num_sms < n_items ? num_sms : n_items);
   if (grid < 1) return cudaSuccess;

@@ -135,12 +135,7 @@ cudaError_t launch_thresholds(const ThrArgs& a, cudaStream_t st) {
   const int threads = 128;
   const int groups = threads / a.n_samples;
   const size_t smem = ((size_t)threads + groups) * a.tb.D * sizeof(float2);
-  int dev = 0, optin = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
-  if (smem > (size_t)optin) return cudaErrorInvalidValue;
-  e = cudaFuncSetAttribute(thresholds_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(thresholds_kernel, smem);
   if (e != cudaSuccess) return e;
   int64_t blocks = (a.count + groups - 1) / groups;
   if (blocks > 152 * 64) blocks = 152 * 64;
