@@ -890,13 +890,13 @@ struct ScanPlan {
 };
 
 rope_status plan_scan(const rope_index* idx, int32_t precision, int64_t n_reads, int64_t jb, int64_t je,
-                      int32_t n_ranges_req, int num_sms, ScanPlan* out, int32_t tc_variant = 0) {
+                      int32_t n_ranges_req, int num_sms, ScanPlan* out, int32_t tc_variant = 0, bool dense = false) {
   const DevIndex& ix = idx->ix;
   if (idx->dense) return fail(ROPE_ERR_UNSUPPORTED, "a materialised index is scored by rope_score_topk / rope_map / rope_score_dense only");
   ScanPlan pl;
   pl.tc = prec_tc(precision);
   int64_t sup;
-  int group, range_group = 0;
+  int group;
   if (pl.tc) {
     if (!scan_tc_supported(ix.D))
       return fail(ROPE_ERR_UNSUPPORTED, "tensor-core scan built for complex dimension 32 or 64, not %d", ix.D);
@@ -909,8 +909,7 @@ rope_status plan_scan(const rope_index* idx, int32_t precision, int64_t n_reads,
     if (!scan_fp32_supported(ix.D))
       return fail(ROPE_ERR_UNSUPPORTED, "FP32 scan built for complex dimension <= 64, not %d", ix.D);
     sup = scan_fp32_super_tile(ix.D);
-    group = scan_fp32_group(ix, n_reads);
-    range_group = scan_fp32_range_group();
+    group = scan_fp32_group();
   } else {
     return fail(ROPE_ERR_INVALID_ARG, "precision %d", precision);
   }
@@ -921,15 +920,15 @@ rope_status plan_scan(const rope_index* idx, int32_t precision, int64_t n_reads,
   a.st0 = (jb / sup) * sup;
   const int64_t n_sup = (je - a.st0 + sup - 1) / sup;
   a.n_groups = (int32_t)((n_reads + group - 1) / group);
-  if (range_group == 0) range_group = group;
-  const int64_t n_rg = (n_reads + range_group - 1) / range_group;
-  int64_t nr = n_ranges_req > 0 ? n_ranges_req : (16LL * num_sms + n_rg - 1) / n_rg;
+  int64_t nr = n_ranges_req > 0 ? n_ranges_req : (16LL * num_sms + a.n_groups - 1) / a.n_groups;
   if (nr < 1) nr = 1;
   if (nr > n_sup) nr = n_sup;
   if (nr > 4096) nr = 4096;
   const int64_t sup_per_range = (n_sup + nr - 1) / nr;
   a.range_len = sup_per_range * sup;
   a.n_ranges = (int32_t)((n_sup + sup_per_range - 1) / sup_per_range);
+  if (!pl.tc && scan_fp32_reads_per_thread(ix, n_reads, a.n_ranges, num_sms, dense) == 2)
+    a.n_groups = (a.n_groups + 1) / 2;
   a.tc_variant = pl.tc ? tc_variant : 0;
   a.fp8 = precision == ROPE_PREC_FP8;
   a.lists_per_range = pl.tc ? scan_tc_lists_per_range(ix.D, a.tc_variant) : 1;
@@ -1520,7 +1519,7 @@ extern "C" rope_status rope_score_dense(const rope_index* idx, const float* emb_
   rope_status st = get_ctx(&c);
   if (st != ROPE_OK) return st;
   ScanPlan pl;
-  if ((st = plan_scan(idx, precision, n_reads, j_begin, j_begin + count, 0, c->num_sms, &pl)) != ROPE_OK) return st;
+  if ((st = plan_scan(idx, precision, n_reads, j_begin, j_begin + count, 0, c->num_sms, &pl, 0, true)) != ROPE_OK) return st;
   pl.a.emb_f32 = emb_f32;
   pl.a.emb_bf16 = emb_bf16;
   pl.a.norms = norms;

@@ -113,8 +113,8 @@ cudaError_t launch_window_embeddings(const DevIndex& ix, int64_t j_begin, int64_
 // rope_scan_fp32.cu
 int scan_fp32_supported(int D);
 int64_t scan_fp32_super_tile(int D);
-int scan_fp32_group(const DevIndex& ix, int64_t n_reads);  // reads per work item
-int scan_fp32_range_group();  // reads per group that the window ranges are laid out for
+int scan_fp32_group();  // reads per group (n_groups) with one read per thread, for which ranges are laid out
+int scan_fp32_reads_per_thread(const DevIndex& ix, int64_t n_reads, int n_ranges, int num_sms, bool dense);
 cudaError_t launch_scan_fp32(const DevIndex& ix, const ScanArgs& a, bool dense, int num_sms, cudaStream_t st);
 
 // rope_scan_tc.cu

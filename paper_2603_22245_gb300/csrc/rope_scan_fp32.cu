@@ -16,6 +16,9 @@
 // 500 reads x 2 M windows (d = 64, 8 candidates): 10.4 ms with one read per
 // thread and unbounded lists, 9.7 ms with two, 8.0 ms with bounded lists; what
 // is left beside the multiply-adds is the updates of each list's first windows.
+// Small calls have neither (256 reads or fewer keep one read per thread, and a
+// block with a single item has no earlier list to bound it by): 256 reads x
+// 500,000 windows 1.66 -> 1.40 ms, 64 reads x 20,000 0.89 -> 0.83 ms.
 #include "rope_internal.h"
 #include "rope_topk.cuh"
 
@@ -56,6 +59,10 @@ template <int D, int R, bool kDense, bool kPerBand>
 __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, ScanArgs a) {
   using Sh = F32Shape<D>;
   constexpr int kGroup = R * kF32Threads;
+  // writing every score at few entries is bound by the stores: 300 reads x 500,000
+  // windows at D = 4 3.5 ms by range, 4.0 ms by group; at D = 32 0.64 and 0.56 ms
+  // (300 reads x 20,000)
+  constexpr bool kByRange = kDense && D < 32;
   static_assert(R == 1 || !kPerBand, "per-band scores take one read per thread");
   extern __shared__ __align__(16) uint8_t f32_smem[];
   float* tile = reinterpret_cast<float*>(f32_smem);
@@ -82,10 +89,22 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
   Chain<D> ch;
   ch.setup(ix, lic);
 
-  // items in group-major order, a contiguous run per block: most of a block's
-  // items share their reads
-  const int it_lo = (int)((int64_t)n_items * blockIdx.x / gridDim.x);
-  const int it_hi = (int)((int64_t)n_items * (blockIdx.x + 1) / gridDim.x);
+  // A contiguous run of items per block. With one read per thread an SM holds two
+  // blocks or more, and the first blocks, which lie on SMs of their own, take the
+  // items left over (4,000 reads x 100,000 windows at D = 16: 2.2 ms, 2.8 ms with
+  // them spread over the blocks); with two it holds one block, and they are spread.
+  // The items are in group-major order, so that most of a block's items share
+  // their reads, or (kByRange) with the groups of a range side by side, so that
+  // full and partly filled groups mix over the SMs.
+  int it_lo, it_hi;
+  if (R == 1) {
+    const int per_block = n_items / (int)gridDim.x, left_over = n_items % (int)gridDim.x;
+    it_lo = (int)blockIdx.x * per_block + min((int)blockIdx.x, left_over);
+    it_hi = it_lo + per_block + ((int)blockIdx.x < left_over ? 1 : 0);
+  } else {
+    it_lo = (int)((int64_t)n_items * blockIdx.x / gridDim.x);
+    it_hi = (int)((int64_t)n_items * (blockIdx.x + 1) / gridDim.x);
+  }
   // Every range has lists of its own, and a list taking its first windows is
   // mostly updates. A list that two earlier lists of the read beat with all
   // their entries cannot add to the merge_depth best of the union, so a window
@@ -96,8 +115,8 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
   int prev_grp = -1;
 
   for (int item = it_lo; item < it_hi; ++item) {
-    const int grp = item / a.n_ranges;
-    const int rng = item % a.n_ranges;
+    const int grp = kByRange ? item % a.n_groups : item / a.n_ranges;
+    const int rng = kByRange ? item / a.n_groups : item % a.n_ranges;
     const int64_t r = (int64_t)grp * kGroup + tid;  // read of slot i: r + i * kF32Threads
     const bool have_read = r < a.n_reads;
     const int64_t st_begin = a.st0 + (int64_t)rng * a.range_len;
@@ -257,7 +276,12 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
 #pragma unroll
                 for (int h = 1; h < kF32Batch; ++h) top = fmaxf(top, sc[i][h]);
                 if (top < lst[i].thr) continue;
-#pragma unroll 1
+                // (with two reads the updates' code, eight times over, costs more than
+                // picking each window's score: 8.8 against 8.0 ms at 500 reads x 2 M
+                // windows; with one read unrolled is the faster, 0.83 against 0.97 ms
+                // at 64 reads x 20,000, but per band, D = 64 and 700 reads x 500,000,
+                // 31 against 26 ms)
+#pragma unroll(R == 1 && !(kPerBand && D == 64) ? kF32Batch : 1)
                 for (int h = 0; h < kF32Batch; ++h) {
                   const int64_t j = jq + h;
                   float v = sc[i][0];
@@ -305,15 +329,26 @@ int64_t scan_fp32_super_tile(int D) {
   return 0;
 }
 
-// Two reads per thread where one group of 256 does not hold them all: a window
-// read from shared memory then serves twice the multiply-adds (see above). At
-// D = 64 two reads' vectors would not fit in registers.
-static int reads_per_thread(const DevIndex& ix, int64_t n_reads) {
-  return ix.D <= 32 && ix.score_mode == 0 && n_reads > kF32Threads ? 2 : 1;
-}
+int scan_fp32_group() { return kF32Threads; }
 
-int scan_fp32_group(const DevIndex& ix, int64_t n_reads) { return kF32Threads * reads_per_thread(ix, n_reads); }
-int scan_fp32_range_group() { return kF32Threads; }
+// Two reads per thread (one generation of a window, and one read of it from
+// shared memory, then serve 512 reads instead of 256) where that pays:
+//   * at D = 32: with fewer entries it was 1.1 to 2.3 times slower almost
+//     throughout, and at D = 64 two reads' vectors do not fit in registers;
+//   * with four items per SM or more, to even out their ends: 500 reads x 1 M windows
+//     (489 items) 5.1 ms against 4.4 with one read, 2,600 x 500,000 (738) 10.3 against
+//     10.9, 500 x 2 M (977) 8.0 against 8.3. Writing every score there are no lists
+//     to fill, and more groups of 256 times ranges than SMs are enough: 1,024 reads x
+//     100,000 1.2 against 1.5 ms, 500 reads 0.95 against 0.57;
+//   * with no half group idle, or a 12th at most: 700 reads x 2 M (three groups of
+//     256) 13.9 against 11.1 ms, 1,100 reads (five) 20.2 against 17.3, 2,600 (eleven)
+//     35.4 against 37.4.
+int scan_fp32_reads_per_thread(const DevIndex& ix, int64_t n_reads, int n_ranges, int num_sms, bool dense) {
+  if (ix.D != 32 || ix.score_mode != 0) return 1;
+  const int64_t g1 = (n_reads + kF32Threads - 1) / kF32Threads, g2 = (g1 + 1) / 2;
+  if (11 * 2 * g2 > 12 * g1) return 1;
+  return (dense ? g1 * n_ranges > num_sms : g2 * n_ranges >= 4 * num_sms) ? 2 : 1;
+}
 
 template <int D, int R, bool kDense, bool kPerBand>
 static cudaError_t launch_one(const DevIndex& ix, const ScanArgs& a, int num_sms, cudaStream_t st) {
@@ -334,22 +369,19 @@ static cudaError_t launch_one(const DevIndex& ix, const ScanArgs& a, int num_sms
   return cudaGetLastError();
 }
 
-template <int D, bool kDense, bool kPerBand>
-static cudaError_t by_reads(const DevIndex& ix, const ScanArgs& a, int num_sms, cudaStream_t st) {
-  if constexpr (D <= 32 && !kPerBand) {
-    if (reads_per_thread(ix, a.n_reads) == 2) return launch_one<D, 2, kDense, kPerBand>(ix, a, num_sms, st);
-  }
-  return launch_one<D, 1, kDense, kPerBand>(ix, a, num_sms, st);
-}
-
 template <bool kDense, bool kPerBand>
 static cudaError_t dispatch(const DevIndex& ix, const ScanArgs& a, int num_sms, cudaStream_t st) {
   switch (ix.D) {
-    case 4: return by_reads<4, kDense, kPerBand>(ix, a, num_sms, st);
-    case 8: return by_reads<8, kDense, kPerBand>(ix, a, num_sms, st);
-    case 16: return by_reads<16, kDense, kPerBand>(ix, a, num_sms, st);
-    case 32: return by_reads<32, kDense, kPerBand>(ix, a, num_sms, st);
-    case 64: return by_reads<64, kDense, kPerBand>(ix, a, num_sms, st);
+    case 4: return launch_one<4, 1, kDense, kPerBand>(ix, a, num_sms, st);
+    case 8: return launch_one<8, 1, kDense, kPerBand>(ix, a, num_sms, st);
+    case 16: return launch_one<16, 1, kDense, kPerBand>(ix, a, num_sms, st);
+    case 32:
+      if constexpr (!kPerBand) {
+        // fewer groups than of 256 reads each: the plan took two reads per thread
+        if ((int64_t)a.n_groups * kF32Threads < a.n_reads) return launch_one<32, 2, kDense, kPerBand>(ix, a, num_sms, st);
+      }
+      return launch_one<32, 1, kDense, kPerBand>(ix, a, num_sms, st);
+    case 64: return launch_one<64, 1, kDense, kPerBand>(ix, a, num_sms, st);
   }
   return cudaErrorInvalidValue;
 }
