@@ -3,6 +3,8 @@
 // the window-embedding inspection kernel.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "rope_internal.h"
 
 namespace rope {
@@ -482,7 +484,15 @@ __device__ __forceinline__ float inv_sqrt_f64(double x) {
 // column = lane (no bank conflicts whatever the bins), sums the first window
 // directly (§2.1-§2.3; stored in FP32, the anchor that seeds the on-chip FP32
 // recurrence) and walks the chunk. The stored 1/sqrt(C_j) thus carries neither
-// the FP32 recurrence's drift nor any rotation's rounding.
+// the FP32 recurrence's drift nor any rotation's rounding. A difference carries
+// the rounding of the largest C it came through, though: four a slide, 256 S a
+// chunk (S letters a window). So a chunk in which C falls by 2^18 / S or more (sums
+// that nearly cancel) is walked a second time, with C formed from the sums wherever
+// it has fallen so far: its relative error stays below 2^-27, an eighth of FP32's.
+// Looking at that in every step of the one walk costs its latency (437 against 420
+// us for 1 Mbp); noting it does not. Where it happens often (one-letter s-mers on a
+// reference with tandem repeats, whose windows cancel wholly) the second walks cost
+// a third more: 323 -> 419 us for 1 Mbp.
 //
 // Bound by the FP64 unit (2 results a cycle per SM): 11 operations a window and
 // band, 2 a location of the first window. A warp per chunk that rotated all D
@@ -511,10 +521,12 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
   const double2* ph = pt.phase + (size_t)k * pt.n_phase;
   const int group = lane - k;
 
-  for (int b = 0; b < nb; ++b) acc[32 * b] = make_double2(0.0, 0.0);
   LetterCursor out, in;  // leaving and entering locations
-  out.start(ix.packed, j0 * S);
-  in.start(ix.packed, j0 * S);
+  double C = 0.0;
+  // high word (ordered as the value, if positive) of the largest C since C was last formed from the sums
+  int peak = 0;
+  const int drop = (18 - (S > 1 ? 32 - __clz(S - 1) : 0)) << 20;
+  bool fallen = false;  // C fell that far below it
   auto bin = [&](LetterCursor& c) { return (uint32_t)__ldg(ix.map_lsb + c.code(s, mask)); };
   auto add = [&](uint32_t b, double2 w) {
     double2 v = acc[32 * b];
@@ -522,7 +534,10 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
     v.y += w.y;
     acc[32 * b] = v;
   };
-  {
+  auto first_window = [&]() {
+    for (int b = 0; b < nb; ++b) acc[32 * b] = make_double2(0.0, 0.0);
+    out.start(ix.packed, j0 * S);
+    in.start(ix.packed, j0 * S);
     int d = 0;
     for (; d + 4 <= n_loc; d += 4) {
       uint32_t b[4];
@@ -536,15 +551,18 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
       for (int q = 0; q < 4; ++q) add(b[q], w[q]);
     }
     for (; d < n_loc; ++d) add(bin(in), __ldg(ph + d));
-  }
-  double C = 0.0;
-  for (int b = 0; b < nb; b += 2) {  // nb = 4^t
-    const double2 v = acc[32 * b], u = acc[32 * (b + 1)];
-    C = fma(v.x, v.x, fma(v.y, v.y, C));
-    C = fma(u.x, u.x, fma(u.y, u.y, C));
-    if (live)
-      *reinterpret_cast<float4*>(anchors + a * ix.D + k * nb + b) = make_float4((float)v.x, (float)v.y, (float)u.x, (float)u.y);
-  }
+  };
+  auto from_sums = [&](bool store) {
+    C = 0.0;
+    for (int b = 0; b < nb; b += 2) {  // nb = 4^t
+      const double2 v = acc[32 * b], u = acc[32 * (b + 1)];
+      C = fma(v.x, v.x, fma(v.y, v.y, C));
+      C = fma(u.x, u.x, fma(u.y, u.y, C));
+      if (store)
+        *reinterpret_cast<float4*>(anchors + a * ix.D + k * nb + b) = make_float4((float)v.x, (float)v.y, (float)u.x, (float)u.y);
+    }
+    peak = __double2hiint(C);
+  };
   const int n_win = (int)min((int64_t)ix.A, ix.W - j0);
   // location d leaves for bin bo, location d + n_loc enters bin bi
   auto slide = [&](uint32_t bo, double2 wo, uint32_t bi, double2 wi) {
@@ -555,9 +573,16 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
     const double q = fma(v.x, wi.x, v.y * wi.y);
     acc[32 * bi] = make_double2(v.x + wi.x, v.y + wi.y);
     C = fma(2.0, q - p, C + 2.0);
+    peak = max(peak, __double2hiint(C));
   };
-  // C of window j over all bands
-  auto total_of = [&](int j) -> double {
+  // C of window j over all bands; exact: formed from the sums where it has fallen
+  auto total_of = [&](int j, bool exact) -> double {
+    const bool low = __double2hiint(C) < peak - drop;
+    if (exact) {
+      if (low) from_sums(false);
+    } else {
+      fallen |= low && j < n_win;
+    }
     double tot = C;
     if (m > 1) {
       tot = 0.0;
@@ -566,43 +591,54 @@ __global__ void prepass_kernel(DevIndex ix, PrepassTables pt, float2* __restrict
     if (band_norm && live && j < n_win) band_norm[(j0 + j) * m + k] = (float)C;
     return tot;
   };
-  for (int jq = 0; jq < kAnchorPeriod; jq += 4) {
-    double tot[4];
-    if (kUnit) {
-      uint32_t bo[4], bi[4];
-      double2 wo[4], wi[4];
+  auto walk = [&](auto exact_c) {
+    constexpr bool exact = decltype(exact_c)::value;
+    for (int jq = 0; jq < kAnchorPeriod; jq += 4) {
+      double tot[4];
+      if (kUnit && !exact) {
+        uint32_t bo[4], bi[4];
+        double2 wo[4], wi[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        bo[q] = bin(out);
-        bi[q] = bin(in);
-        // (the slide after the chunk's last window is not needed)
-        const int d = min(jq + q, kAnchorPeriod - 2);
-        wo[q] = __ldg(ph + d);
-        wi[q] = __ldg(ph + d + n_loc);
-      }
+        for (int q = 0; q < 4; ++q) {
+          bo[q] = bin(out);
+          bi[q] = bin(in);
+          // (the slide after the chunk's last window is not needed)
+          const int d = min(jq + q, kAnchorPeriod - 2);
+          wo[q] = __ldg(ph + d);
+          wi[q] = __ldg(ph + d + n_loc);
+        }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        tot[q] = total_of(jq + q);
-        slide(bo[q], wo[q], bi[q], wi[q]);
-      }
-    } else {
+        for (int q = 0; q < 4; ++q) {
+          tot[q] = total_of(jq + q, exact);
+          slide(bo[q], wo[q], bi[q], wi[q]);
+        }
+      } else {
 #pragma unroll 1
-      for (int q = 0; q < 4; ++q) {
-        const double v = total_of(jq + q);
-        tot[0] = q == 0 ? v : tot[0];
-        tot[1] = q == 1 ? v : tot[1];
-        tot[2] = q == 2 ? v : tot[2];
-        tot[3] = q == 3 ? v : tot[3];
-        if (jq + q == kAnchorPeriod - 1) break;
-        const int d0 = (jq + q) * S;
-        for (int u = 0; u < S; ++u) slide(bin(out), __ldg(ph + d0 + u), bin(in), __ldg(ph + d0 + u + n_loc));
+        for (int q = 0; q < 4; ++q) {
+          const double v = total_of(jq + q, exact);
+          tot[0] = q == 0 ? v : tot[0];
+          tot[1] = q == 1 ? v : tot[1];
+          tot[2] = q == 2 ? v : tot[2];
+          tot[3] = q == 3 ? v : tot[3];
+          if (jq + q == kAnchorPeriod - 1) break;
+          const int d0 = (jq + q) * S;
+          for (int u = 0; u < S; ++u) slide(bin(out), __ldg(ph + d0 + u), bin(in), __ldg(ph + d0 + u + n_loc));
+        }
+      }
+      // the four roots are shared among the chunk's lanes (each knows all totals)
+      for (int q = k; q < 4; q += m) {
+        const double v = q < 2 ? (q == 0 ? tot[0] : tot[1]) : (q == 2 ? tot[2] : tot[3]);
+        if (live && jq + q < n_win) inv_norm[j0 + jq + q] = v > (double)kZeroNorm2 ? inv_sqrt_f64(v) : 0.f;
       }
     }
-    // the four roots are shared among the chunk's lanes (each knows all totals)
-    for (int q = k; q < 4; q += m) {
-      const double v = q < 2 ? (q == 0 ? tot[0] : tot[1]) : (q == 2 ? tot[2] : tot[3]);
-      if (live && jq + q < n_win) inv_norm[j0 + jq + q] = v > (double)kZeroNorm2 ? inv_sqrt_f64(v) : 0.f;
-    }
+  };
+  first_window();
+  from_sums(live);
+  walk(std::false_type());
+  if (__any_sync(0xffffffffu, fallen)) {
+    first_window();
+    from_sums(false);
+    walk(std::true_type());
   }
 }
 
