@@ -265,16 +265,19 @@ rope_status rope_noalloc_sync_status(cudaStream_t stream);
  * length, read groups and scanned windows rounded up to powers of two,
  * cand_depth, sep on/off) with opts->n_ranges == 0, the library times each
  * variant with 8, 16 and 32 items per SM on that call's reads and windows and
- * keeps the fastest for the class; later calls of the class use it. Only
+ * keeps the fastest for the class (for windows past 2,048 letters the third
+ * variant unless another is faster by 15%); later calls of the class use it. Only
  * scans of at most 2^22 windows are timed (short samples of a longer scan
  * mispredict it: the cost per window falls with the scan's length); longer
  * ones keep the defaults (variant 0, 16 items per SM) unless set by hand.
- * Results do not depend on the choice.
+ * Window scores do not depend on the choice, nor do results where cand_depth is
+ * at least rescore_depth; with shallower lists (the defaults) the last entries of
+ * a read's results may, as the choice decides which windows share a list.
  * Tuning is on unless the environment sets ROPE_AUTOTUNE=0; the
  * allocation-free entry point only reads earlier choices. */
 rope_status rope_autotune_enable(int32_t enabled);  /* 0 also forgets earlier choices */
 /* Records (variant, items per SM) for the class of (idx, n_reads, opts), as if
- * tuned: later calls of the class use it. variant < 2 at d = 64, 0 at d = 128. */
+ * tuned: later calls of the class use it. variant < 3 at d = 64, 0 at d = 128. */
 rope_status rope_autotune_set(const rope_index* idx, int64_t n_reads, const rope_score_opts* opts, int32_t variant,
                               int32_t items_per_sm);
 /* The choice recorded for the class of (idx, n_reads, opts): tile variant,

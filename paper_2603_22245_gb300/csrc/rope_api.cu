@@ -961,10 +961,17 @@ rope_status check_opts(const rope_score_opts* o, rope_score_opts* v) {
 // a shape class (device, complex dimension, stride, window length and read
 // groups to the nearest power of two, candidate depth, sep on/off) the tuner
 // times every (variant, items per SM) pair on a sample of the call's own
-// windows with the call's own reads and keeps the fastest for that class. The
-// results of a scan do not depend on these choices (each window's score is
-// the same product; the merge takes the best entries of all lists), only its
-// speed does. ROPE_AUTOTUNE=0 (or rope_autotune_enable(0)) keeps the defaults.
+// windows with the call's own reads and keeps the fastest for that class.
+// ROPE_AUTOTUNE=0 (or rope_autotune_enable(0)) keeps the defaults.
+//
+// A window's score does not depend on these choices. What the merge takes depends
+// on them only with re-scoring and lists shallower than it (cand_depth below
+// rescore_depth; the defaults are 8 and 16 at k = 8): an entry among a read's 16
+// best is then missing if eight better ones lie in the same list, and which
+// windows share a list differs by variant and split. At k = 8 the variants' results
+// differed in up to 2 of 9,600 entries at windows of up to 2,000 letters and
+// stride 8, 5 of 3,200 at 4,149, 5 of 9,600 at 10,000 (89 of 9,600 there at stride
+// 1); with cand_depth 16 in none.
 
 struct TuneKey {
   int dev, D, stride, n_log2, g_log2, w_log2, cand_depth, sep_on, fp8;
@@ -1107,12 +1114,14 @@ rope_status tune_tc(const rope_index* idx, const uint16_t* emb_bf16, const float
       any = true;
     }
   }
-  // Long windows overlap almost entirely, so a read's 8 kept and 16 re-scored
-  // candidates are near-equal neighbours and the last of its results can move
-  // with the split of the windows over lists, which differs by variant. There
-  // (and with more than one group of reads) the 512-read variant is kept unless
-  // another is clearly faster: at 4,149 letters and 581 reads the two are 0.76
-  // and 0.70 ms, at 672 letters and 319 reads 0.38 and 0.48 ms.
+  // A rule about results, not speed: long windows overlap almost entirely, so a
+  // read's best candidates are near-equal neighbours and the last of its results
+  // moves with the variant most often there (see above), while the variants' times
+  // lie so close that noise would choose between them from process to process.
+  // There (and with more than one group of reads) the 512-read variant is kept
+  // unless another is faster by 15%. At 3,000 to 10,000 letters and stride 8 it is
+  // the fastest with 400 and 1,200 reads and 3-6% slower than the fastest with 600;
+  // at stride 1 and 1,200 reads it is 5-7% slower.
   if (scan_tc_variants(ix.D) == 3 && ix.N > 2048 && n_groups(0) > 1 && by_variant[2].sample_ms < 1.15f * b.sample_ms)
     b = by_variant[2];
   cudaEventDestroy(e0);
