@@ -44,7 +44,7 @@ namespace rope {
 // the normal range of E4M3, except for entries near 0.
 constexpr float kFp8Scale = 32.f;
 
-template <int D_, int NT_, int T_, int NB_, int LPC_, int EW_, int LH_, int NM_, bool ISOLATE_MMA_, bool FP8_ = false>
+template <int D_, int NT_, int T_, int NB_, int LPC_, int EW_, int NM_, bool ISOLATE_MMA_, bool FP8_ = false>
 struct TcShape {
   static constexpr int D = D_, NT = NT_, T = T_, NB = NB_;  // NB: most B ring slots
   static constexpr int A = kAnchorPeriod;
@@ -53,8 +53,7 @@ struct TcShape {
   static constexpr int CPW = 32 / LPC;           // chains per warp
   static constexpr int GEN_WARPS = T / CPW;
   static constexpr int EW = EW_;                 // epilogue warps sharing one accumulator's columns
-  static constexpr int LH = LH_;                 // candidate lists per read (column halves)
-  static constexpr int LPW = LH / EW;            // lists per epilogue warp
+  static constexpr int LH = EW;                  // candidate lists per read: one per warp's share of the columns
   static constexpr int WPH = T / EW;             // windows per epilogue warp per stage
   static constexpr int EPI_WARPS = 4 * NT * EW;
   // Roles after the epilogue warps: a bin warp, NM MMA-issuing warps and the
@@ -119,7 +118,7 @@ struct TcShape {
   static_assert(GEN_WARPS * CPW == T, "T must be a multiple of chains per warp");
   static_assert((NM == 2 || NM == 4) && NM % NT == 0 && (NM == NT || NM == NT * STG) && STG >= 1 && STG * NT * 2 * T <= TMEM_COLS, "tensor memory budget");
   static_assert(A % STEP == 0, "every item starts at the first of a tile's issuers");
-  static_assert(WPH % 16 == 0 && LPW >= 1 && (LPW == 1 || WPH % (16 * LPW) == 0), "the epilogue loads 16-column chunks");
+  static_assert(WPH % 16 == 0, "the epilogue loads 16-column chunks");
   static_assert(BPL * EB == 8 || (BPL * EB) % 16 == 0, "generator lanes write 8-byte or whole 16-byte pieces");
   static_assert(KBLK == 64 || KBLK == 128, "swizzle row");
   static_assert((2 * T) % 16 == 0 && 2 * T <= 256, "MMA N");
@@ -187,8 +186,8 @@ __device__ __forceinline__ float max_abs2(const uint32_t (&vr)[16], const uint32
 // updates: a list's content is the best of all offered, whatever the order.
 //
 // Per epilogue lane, words at a stride of QS bytes (the block's epilogue lanes):
-// a head (count in bits 0-7, worst entry of list l in bits 8+8l..15+8l), then
-// the entries' (score, window) pairs.
+// a head (count in bits 0-7, the list's worst entry in bits 8-15), then the
+// entries' (score, window) pairs.
 constexpr int kPend = 4;  // most entries (fewer where shared memory is short)
 constexpr int queue_words(int pend) { return 1 + 2 * pend; }
 
@@ -202,41 +201,33 @@ __device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) { asm volatile("
 // What the out-of-line part of the epilogue needs besides its arguments.
 struct ListRef {
   uint32_t queue;    // this lane's queue
-  uint32_t lists;    // this lane's first list (scores; list l: + 4 l GROUP bytes)
-  uint32_t win_off;  // from a list's scores to its windows, bytes
+  uint32_t list;     // this lane's list (scores)
+  uint32_t win_off;  // from its scores to its windows, bytes
   int32_t depth, sep, stride, pend;
 };
 
-// The queued candidates into their lists; head: the queue's head word, thr: each
-// list's worst score. With two lists the window's half of the stage's columns
-// (bit HALF_SHIFT of its number) picks the list. Leaves the queue empty.
+// The queued candidates into the list; head: the queue's head word, thr: the
+// list's worst score. Leaves the queue empty.
 template <class Sh>
-__device__ __forceinline__ void flush_queue(const ListRef& q, uint32_t& head, float (&thr)[Sh::LPW]) {
+__device__ __forceinline__ void flush_queue(const ListRef& q, uint32_t& head, float& thr) {
   constexpr uint32_t QS = 4u * Sh::GROUP * Sh::EW;
-  constexpr int HALF_SHIFT = Sh::SUP == 4096 ? 11 : 10;
   const uint32_t cnt = head & 0xFFu;
   const uint32_t n = __reduce_max_sync(0xffffffffu, cnt);
   for (uint32_t e = 0; e < n; ++e) {
     if (e < cnt) {
       const float v = __uint_as_float(lds_u32(q.queue + (1 + 2 * e) * QS));
       const uint32_t j = lds_u32(q.queue + (2 + 2 * e) * QS);
-      const uint32_t l = Sh::LPW == 2 ? (j >> HALF_SHIFT) & 1u : 0u;
-      const float th = Sh::LPW == 2 && l ? thr[Sh::LPW - 1] : thr[0];
-      if (v >= th) {
+      if (v >= thr) {
         ThreadList tl;
-        tl.s = static_cast<float*>(__cvta_shared_to_generic(q.lists + 4 * l * Sh::GROUP));
-        tl.w = static_cast<uint32_t*>(__cvta_shared_to_generic(q.lists + 4 * l * Sh::GROUP + q.win_off));
+        tl.s = static_cast<float*>(__cvta_shared_to_generic(q.list));
+        tl.w = static_cast<uint32_t*>(__cvta_shared_to_generic(q.list + q.win_off));
         tl.stride = Sh::GROUP * Sh::LH;
         tl.depth = q.depth;
-        tl.worst = (int)((head >> (8 + 8 * l)) & 0xFFu);
-        tl.thr = th;
+        tl.worst = (int)((head >> 8) & 0xFFu);
+        tl.thr = thr;
         tl.insert(v, j, q.sep, q.stride);
-        head = (head & ~(0xFFu << (8 + 8 * l))) | ((uint32_t)tl.worst << (8 + 8 * l));
-        if (Sh::LPW == 2 && l) {
-          thr[Sh::LPW - 1] = tl.thr;
-        } else {
-          thr[0] = tl.thr;
-        }
+        head = (head & ~0xFF00u) | ((uint32_t)tl.worst << 8);
+        thr = tl.thr;
       }
     }
     __syncwarp();
@@ -246,10 +237,7 @@ __device__ __forceinline__ void flush_queue(const ListRef& q, uint32_t& head, fl
 
 // Every queued candidate into its list (the end of a read group).
 template <class Sh>
-__device__ __noinline__ void flush_all(ListRef q, float thr0, float thr1) {
-  float thr[Sh::LPW];
-  thr[0] = thr0;
-  if (Sh::LPW == 2) thr[Sh::LPW - 1] = thr1;
+__device__ __noinline__ void flush_all(ListRef q, float thr) {
   uint32_t head = lds_u32(q.queue);
   flush_queue<Sh>(q, head, thr);
 }
@@ -261,15 +249,12 @@ __device__ __noinline__ void flush_all(ListRef q, float thr0, float thr1) {
 // Out of line, and its state in shared memory, so that the hot loop holds few
 // registers and spills none: a block's local memory exceeds the L1 that its
 // shared memory leaves, so a reload in that loop would cost an L2 round trip.
-// jc0: window of the share's first column. Returns the new thresholds.
+// jc0: window of the share's first column. Returns the new threshold.
 template <class Sh>
-__device__ __noinline__ float2 offer_chunks(ListRef q, uint32_t tcol, uint32_t todo, uint32_t jc0, uint32_t jlo,
-                                            uint32_t jhi, float thr0, float thr1, uint64_t* bar_empty) {
+__device__ __noinline__ float offer_chunks(ListRef q, uint32_t tcol, uint32_t todo, uint32_t jc0, uint32_t jlo,
+                                           uint32_t jhi, float thr, uint64_t* bar_empty) {
   constexpr uint32_t QS = 4u * Sh::GROUP * Sh::EW;
   constexpr int A = Sh::A;
-  float thr[Sh::LPW];
-  thr[0] = thr0;
-  if (Sh::LPW == 2) thr[Sh::LPW - 1] = thr1;
   uint32_t head = lds_u32(q.queue);
   while (todo) {
     const int c0 = 16 * (__ffs(todo) - 1);
@@ -286,13 +271,12 @@ __device__ __noinline__ float2 offer_chunks(ListRef q, uint32_t tcol, uint32_t t
       __syncwarp();
       if ((threadIdx.x & 31) == 0) mbar_arrive(bar_empty);
     }
-    const float th = Sh::LPW == 2 && c0 >= Sh::WPH / 2 ? thr[Sh::LPW - 1] : thr[0];
     float sc[16];
 #pragma unroll
     for (int n = 0; n < 16; n += 2) abs2_pair(vr[n], vr[n + 1], vi[n], vi[n + 1], sc[n], sc[n + 1]);
     uint32_t pass = 0;  // the windows at or above the threshold
 #pragma unroll
-    for (int n = 0; n < 16; ++n) pass |= sc[n] >= th ? (1u << n) : 0u;
+    for (int n = 0; n < 16; ++n) pass |= sc[n] >= thr ? (1u << n) : 0u;
     while (__any_sync(0xffffffffu, pass != 0)) {
       while (pass != 0 && (head & 0xFFu) < (uint32_t)q.pend) {
         const int n = __ffs(pass) - 1;
@@ -312,7 +296,7 @@ __device__ __noinline__ float2 offer_chunks(ListRef q, uint32_t tcol, uint32_t t
     }
   }
   sts_u32(q.queue, head);
-  return make_float2(thr[0], thr[Sh::LPW - 1]);
+  return thr;
 }
 
 // kDense: every score written to a.dense. kThr: every score at or above its
@@ -322,7 +306,7 @@ template <class Sh, bool kDense, bool kThr = false>
 __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, ScanArgs a, TcLaunch L) {
   constexpr bool kLists = !kDense && !kThr;
   constexpr int D = Sh::D, NT = Sh::NT, T = Sh::T, NB = Sh::NB, A = Sh::A, BPL = Sh::BPL;
-  constexpr int NACC = Sh::NACC, STG = Sh::STG, LPW = Sh::LPW;
+  constexpr int NACC = Sh::NACC, STG = Sh::STG;
   extern __shared__ __align__(1024) uint8_t tc_smem_raw[];
   __shared__ __align__(8) uint64_t bar_bfull[NB], bar_bempty[NB];
   __shared__ __align__(8) uint64_t bar_afull[NACC], bar_aempty[NACC];
@@ -402,8 +386,7 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
   if (warp < Sh::EPI_WARPS) {
     // ================================================================ epilogue
     // warp = (share w, tile, lane quarter q); share w holds windows
-    // [w*WPH, (w+1)*WPH) of each stage and LPW candidate lists per read over
-    // equal parts of them.
+    // [w*WPH, (w+1)*WPH) of each stage and a candidate list per read over them.
     const int q = warp & 3;
     const int tile = (warp >> 2) % NT;
     const int w = warp / (4 * NT);
@@ -414,19 +397,16 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
     uint32_t use = 0;      // accumulators of this tile consumed
     int prev_grp = -1;     // read group of the list being kept
     int seg_rng = 0;       // range whose slot receives that list
-    // thresholds: each list's worst kept score (+inf for a missing read, whose lists take nothing)
-    float thr0 = INFINITY, thr1 = INFINITY;
-    const ListRef lref{smem_u32(queues + w * Sh::GROUP + rs), smem_u32(list_s + w * LPW * Sh::GROUP + rs),
+    // threshold: the list's worst kept score (+inf for a missing read, whose list takes nothing)
+    float thr_list = INFINITY;
+    const ListRef lref{smem_u32(queues + w * Sh::GROUP + rs), smem_u32(list_s + w * Sh::GROUP + rs),
                        4u * a.cand_depth * Sh::GROUP * Sh::LH, a.cand_depth, a.sep, S, L.pend};
-    // writes the kept lists of read r to the slots of range rng
+    // writes the kept list of read r to the slot of range rng
     auto flush = [&](int64_t r, int rng) {
-      const float* ls = list_s + w * LPW * Sh::GROUP + rs;
-      const uint32_t* lw = list_w + w * LPW * Sh::GROUP + rs;
-      for (int l = 0; l < LPW; ++l) {
-        Candidate* out = a.cand + (((size_t)r * a.n_ranges + rng) * Sh::LH + w * LPW + l) * a.cand_depth;
-        for (int e = 0; e < a.cand_depth; ++e)
-          out[e] = Candidate{ls[e * lstride + l * Sh::GROUP] * Sh::SCORE_SCALE, lw[e * lstride + l * Sh::GROUP]};
-      }
+      const float* ls = list_s + w * Sh::GROUP + rs;
+      const uint32_t* lw = list_w + w * Sh::GROUP + rs;
+      Candidate* out = a.cand + (((size_t)r * a.n_ranges + rng) * Sh::LH + w) * a.cand_depth;
+      for (int e = 0; e < a.cand_depth; ++e) out[e] = Candidate{ls[e * lstride] * Sh::SCORE_SCALE, lw[e * lstride]};
     };
     for (int64_t item = it_lo; item < it_hi; ++item) {
       const int grp = (int)(item / a.n_ranges);
@@ -445,7 +425,7 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
         // tile have all completed: its warps consumed every accumulator.
         if (kLists && prev_grp >= 0) {
           const int64_t pr = (int64_t)prev_grp * Sh::GROUP + rs;
-          flush_all<Sh>(lref, thr0, thr1);
+          flush_all<Sh>(lref, thr_list);
           if (pr < a.n_reads) flush(pr, seg_rng);
         }
         if (w == 0) {
@@ -467,23 +447,21 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
           }
           fence_proxy_async_smem();
         }
-        thr0 = thr1 = have_read ? -INFINITY : INFINITY;
+        thr_list = have_read ? -INFINITY : INFINITY;
         if (kLists) {
           sts_u32(lref.queue, 0u);
-          float* ls = list_s + w * LPW * Sh::GROUP + rs;
-          uint32_t* lw = list_w + w * LPW * Sh::GROUP + rs;
-          for (int e = 0; e < a.cand_depth; ++e)
-            for (int l = 0; l < LPW; ++l) {
-              ls[e * lstride + l * Sh::GROUP] = -INFINITY;
-              lw[e * lstride + l * Sh::GROUP] = kEmptyWin;
-            }
+          float* ls = list_s + w * Sh::GROUP + rs;
+          uint32_t* lw = list_w + w * Sh::GROUP + rs;
+          for (int e = 0; e < a.cand_depth; ++e) {
+            ls[e * lstride] = -INFINITY;
+            lw[e * lstride] = kEmptyWin;
+          }
         }
         prev_grp = grp;
         seg_rng = rng;
       } else if (kLists && have_read) {
         // the list carries on: this range's own slot holds no list
-        for (int l = 0; l < LPW; ++l)
-          a.cand[(((size_t)r * a.n_ranges + rng) * Sh::LH + w * LPW + l) * a.cand_depth].win = kUnusedWin;
+        a.cand[(((size_t)r * a.n_ranges + rng) * Sh::LH + w) * a.cand_depth].win = kUnusedWin;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_aready);
@@ -524,15 +502,12 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
               reg_fence(vr);
               reg_fence(vi);
               reg_fence(mr, mi);
-              const float th = LPW == 2 && u >= NCH / 2 ? thr1 : thr0;
-              if (__any_sync(0xffffffffu, fmaf(mr, mr, mi * mi) >= th)) todo |= max_abs2(vr, vi) >= th ? 1u << u : 0u;
+              if (__any_sync(0xffffffffu, fmaf(mr, mr, mi * mi) >= thr_list)) todo |= max_abs2(vr, vi) >= thr_list ? 1u << u : 0u;
             }
             if (__any_sync(0xffffffffu, todo != 0)) {
               todo = __reduce_or_sync(0xffffffffu, todo);
-              const float2 t = offer_chunks<Sh>(lref, tcol, todo, jbase + (uint32_t)(w * Sh::WPH * A), jlo, jhi, thr0,
-                                                thr1, &bar_aempty[acc]);
-              thr0 = t.x;
-              thr1 = t.y;
+              thr_list = offer_chunks<Sh>(lref, tcol, todo, jbase + (uint32_t)(w * Sh::WPH * A), jlo, jhi, thr_list,
+                                      &bar_aempty[acc]);
             } else {
               // nothing to offer: hand the accumulator back
               tc_fence_before();
@@ -613,7 +588,7 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
     }
     if (kLists && prev_grp >= 0) {
       const int64_t pr = (int64_t)prev_grp * Sh::GROUP + rs;
-      flush_all<Sh>(lref, thr0, thr1);
+      flush_all<Sh>(lref, thr_list);
       if (pr < a.n_reads) flush(pr, seg_rng);
     }
   epi_done:;
@@ -908,24 +883,24 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
 //          generators and MMAs; 29 warps of 64 registers. With 8 epilogue warps
 //          (two lists each, 80 registers) 407 instead of 370 ms on 16,384 reads x
 //          100 M windows; with two issuers (27 warps of 72 registers) 440 ms.
-using TcShape32 = TcShape<32, 2, 64, 6, 4, 2, 2, 4, false>;
+using TcShape32 = TcShape<32, 2, 64, 6, 4, 2, 4, false>;
 // d = 64, second tile variant: one epilogue warp per accumulator quarter and
 //          tile (8 warps, each reading all 64 windows of a stage; one candidate
 //          list per read), more registers per thread. Faster at large strides.
-using TcShape32b = TcShape<32, 2, 64, 4, 4, 1, 1, 4, true>;
+using TcShape32b = TcShape<32, 2, 64, 4, 4, 1, 4, true>;
 // d = 64, third tile variant: 512 reads (4 tiles) x 32 windows per stage, MMA
 //          N = 64 (twice the MMA instructions per score), super-tiles of half
 //          the windows: a finer split of short references.
-using TcShape32c = TcShape<32, 4, 32, 4, 4, 1, 1, 4, false>;
+using TcShape32c = TcShape<32, 4, 32, 4, 4, 1, 4, false>;
 // d = 128: 256 reads x 64 windows per stage, MMA N = 128 (twice the tensor time
 //          per stage); 8 epilogue warps, 16 generator warps (chains of 8 lanes x 8 entries)
-using TcShape64 = TcShape<64, 2, 64, 2, 8, 1, 1, 2, false>;
+using TcShape64 = TcShape<64, 2, 64, 2, 8, 1, 2, false>;
 // the same tiles with E4M3 operands (kind::f8f6f4): half the operand bytes,
 // half the MMA instructions per stage; 64-byte swizzled rows at d = 64
-using TcShape32f8 = TcShape<32, 2, 64, 4, 4, 2, 2, 4, false, true>;
-using TcShape32bf8 = TcShape<32, 2, 64, 4, 4, 1, 1, 4, true, true>;
-using TcShape32cf8 = TcShape<32, 4, 32, 4, 4, 1, 1, 4, false, true>;
-using TcShape64f8 = TcShape<64, 2, 64, 2, 8, 1, 1, 2, false, true>;
+using TcShape32f8 = TcShape<32, 2, 64, 4, 4, 2, 4, false, true>;
+using TcShape32bf8 = TcShape<32, 2, 64, 4, 4, 1, 4, true, true>;
+using TcShape32cf8 = TcShape<32, 4, 32, 4, 4, 1, 4, false, true>;
+using TcShape64f8 = TcShape<64, 2, 64, 2, 8, 1, 2, false, true>;
 
 // Dynamic shared memory one block of this kernel may take: the device's
 // opt-in maximum per block less the kernel's static shared memory (barriers,
@@ -1001,7 +976,7 @@ static size_t tc_smem_bytes(const DevIndex& ix, int cand_depth, bool lists, int 
 
 // The same tiles with one MMA issuer per read tile, for a ring of one slot.
 template <class Sh>
-using TcOneSlot = TcShape<Sh::D, Sh::NT, Sh::T, 1, Sh::LPC, Sh::EW, Sh::LH, Sh::NT, Sh::ISOLATE_MMA, Sh::FP8>;
+using TcOneSlot = TcShape<Sh::D, Sh::NT, Sh::T, 1, Sh::LPC, Sh::EW, Sh::NT, Sh::ISOLATE_MMA, Sh::FP8>;
 
 // The most B slots, with two buffers of bins before one and whole queues before
 // shorter ones, that fit in `limit` bytes; 0 if none do. Where a tile has two MMA
