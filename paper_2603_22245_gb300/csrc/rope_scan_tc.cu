@@ -29,7 +29,7 @@
 // of its tensor-memory loads) is what the rest waits for. Measured on that case
 // and on 16,384 reads x 100 M windows, against one issuing thread, a bin fill by
 // the generators, scores formed for every column and list updates before the
-// hand-over (236 ms and 553 ms): 167 ms and 370 ms.
+// hand-over (234 ms and 553 ms): 171 ms and 385 ms.
 // Every wait is bounded; a wait that runs out sets the timeout status bit and
 // the block drains its in-flight copies and MMAs, frees tensor memory and exits.
 #include <cuda_bf16.h>
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
             // thresholds of all 32 reads costs two loads and three operations
             // instead of the 16 scores and their maximum. A bound that reaches a
             // threshold is looked at exactly (the columns are in registers).
-            // Forming every score measured 437 ms, this 370 ms (16,384 reads x
+            // Forming every score measured 450 ms, this 385 ms (16,384 reads x
             // 100 M windows); with lists of under ~10^6 windows, where half of
             // the bounds pass, the two are equal.
             constexpr int NCH = Sh::WPH / 16;
@@ -881,8 +881,8 @@ __global__ void __launch_bounds__(Sh::NTHREADS, 1) scan_tc_kernel(DevIndex ix, S
 //          per accumulator quarter, a list each), 8 generator warps (chains of 4
 //          lanes x 8 entries), four issuers, up to 6 window slots between
 //          generators and MMAs; 29 warps of 64 registers. With 8 epilogue warps
-//          (two lists each, 80 registers) 407 instead of 370 ms on 16,384 reads x
-//          100 M windows; with two issuers (27 warps of 72 registers) 440 ms.
+//          (the second variant) 416 instead of 385 ms on 16,384 reads x 100 M
+//          windows; with two issuers (27 warps of 72 registers) 445 ms.
 using TcShape32 = TcShape<32, 2, 64, 6, 4, 2, 4, false>;
 // d = 64, second tile variant: one epilogue warp per accumulator quarter and
 //          tile (8 warps, each reading all 64 windows of a stage; one candidate
