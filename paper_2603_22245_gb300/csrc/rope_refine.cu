@@ -155,6 +155,12 @@ __device__ __forceinline__ uint32_t packed_code(const uint32_t* __restrict__ pac
   return ((g & 0x55555555u) << 1) | ((g >> 1) & 0x55555555u);
 }
 
+// Whether fidelity f beats g by more than the rounding of the FP64 sums they come
+// from: positions that are equal but for it are ties, which go to the lower one
+// (an s-mer that a read shares with a range gives the same fidelity half a window
+// further on).
+__device__ __forceinline__ bool ref_beats(double f, double g) { return f > fma(g, 1e-12, g) + 1e-20; }
+
 // |v|^2 in FP64 (the products of FP32 values are exact)
 __device__ __forceinline__ double norm2(float2 v) { return (double)v.x * v.x + (double)v.y * v.y; }
 
@@ -420,25 +426,18 @@ __global__ void __launch_bounds__(256) refine_kernel(RefineArgs a) {
         }
         if (t < n_steps) {
           const double f = fid_at(t + 1, jr, ji, ck);
-          if (f > best) {
-            best = f;
-            best_i = t + 1;
-          }
+          if (ref_beats(f, best)) best_i = t + 1;
+          best = fmax(best, f);
         }
       }
-      // the best position, ties to the lower
+      // the best fidelity, and the lowest position that it does not beat
+      double top = best;
 #pragma unroll
-      for (int w = 16; w > 0; w >>= 1) {
-        const double f = __shfl_xor_sync(0xffffffffu, best, w);
-        const int i = __shfl_xor_sync(0xffffffffu, best_i, w);
-        if (f > best || (f == best && i < best_i)) {
-          best = f;
-          best_i = i;
-        }
-      }
+      for (int w = 16; w > 0; w >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, w));
+      best_i = (int)__reduce_min_sync(0xffffffffu, ref_beats(top, best) ? 0x7FFFFFFFu : (unsigned)best_i);
       if (lane == 0) {
         a.out_pos[o] = p0 + best_i;
-        a.out_fid[o] = (float)best;
+        a.out_fid[o] = (float)top;
       }
       __syncwarp();  // the tables are free for the next candidate
     }
