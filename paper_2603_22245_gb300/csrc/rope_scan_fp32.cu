@@ -90,9 +90,10 @@ __global__ void __launch_bounds__(kF32Threads) scan_fp32_kernel(DevIndex ix, Sca
   ch.setup(ix, lic);
 
   // A contiguous run of items per block. With one read per thread an SM holds two
-  // blocks or more, and the first blocks, which lie on SMs of their own, take the
-  // items left over (4,000 reads x 100,000 windows at D = 16: 2.2 ms, 2.8 ms with
-  // them spread over the blocks); with two it holds one block, and they are spread.
+  // blocks or more (but at D = 64), and the first blocks, which lie on SMs of their
+  // own, take the items left over (4,000 reads x 100,000 windows at D = 16: 2.2 ms,
+  // 2.8 ms with them spread over the blocks); with two it holds one block, and they
+  // are spread (1,000 reads x 8 M at D = 32: 48.1 ms, 49.1 ms with the first blocks).
   // The items are in group-major order, so that most of a block's items share
   // their reads, or (kByRange) with the groups of a range side by side, so that
   // full and partly filled groups mix over the SMs.

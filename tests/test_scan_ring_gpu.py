@@ -1,7 +1,7 @@
 """The tensor-core scan with few window slots: deep candidate lists, large
 strides and long windows leave shared memory for two slots and a short queue of
-candidates, for one buffer of bins, or for a single slot, which one of a read
-tile's two MMA issuers serves alone."""
+candidates, for one buffer of bins, or for a single slot, where each read tile has
+one MMA issuer instead of two."""
 import numpy as np
 import pytest
 import torch
